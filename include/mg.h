@@ -85,10 +85,11 @@ typedef enum { MG_MEM_HOST = 0, MG_MEM_DEVICE = 1 } mg_mem;
  *                  eta^inner_cycles (eta per multigrid iteration).
  *  coarse_cluster  1 = run the middle coarse levels (4096 to 131072 cells per
  *                  colour) and the bottom levels of a V-cycle as one launch of
- *                  one thread-block cluster; 0 = one launch per step (faster
- *                  on GB300: the replayed graph pipelines the launches, while
- *                  each cluster-wide step costs a barrier).  The results are
- *                  the same.
+ *                  one thread-block cluster, through global memory; 0 = the
+ *                  coarse levels that fit the shared memory of a cluster run
+ *                  from there as one launch (n_pre, n_post >= 1), the ones
+ *                  above them one launch per step (faster on GB300).  The
+ *                  results are the same.
  *  smoother_pass   mixed form: 1 = run each pair of FP32 Gauss-Seidel sweeps
  *                  of the fine level (N_pre = N_post = 2 is one pair) as one
  *                  temporal-blocked pass over the level (a z-wavefront over

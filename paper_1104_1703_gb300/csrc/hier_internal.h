@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "../../include/mg.h"
+#include "cluster_internal.h"
 #include "mg_internal.h"
 #include "pass_internal.h"
 
@@ -71,7 +72,20 @@ struct mg_hierarchy {
   int max_partials = 0;
   double* dscal = nullptr;             // device scalars
   int* err_flag = nullptr;
+  // What a mask build tells the host, contiguous in the arena and copied to
+  // pinned memory at once: counts, every level's list counts, plane starts.
   unsigned long long* counts = nullptr;  // [kMaxLevels][2]
+  char* build_info = nullptr;
+  size_t build_info_bytes = 0;
+  const char* hbuild_info = nullptr;  // its pinned copy
+  // the coarse levels' cluster launch per order (first level 0: none) and its
+  // record blobs, and a hash of the list lengths and plane starts (captured
+  // graphs depend on them)
+  bool cluster_ok = false;
+  gbmg::ClPlan cl_plan[3];
+  char* cl_blobs[3] = {nullptr, nullptr, nullptr};
+  size_t cl_bound = 0;
+  unsigned long long lists_hash = 0;
   double* hscal = nullptr;               // pinned host scalars
   void* staging = nullptr;
   size_t staging_bytes = 0;

@@ -512,6 +512,21 @@ __global__ void __launch_bounds__(kListThreads) list_write_all_kernel(const List
   for (unsigned i = threadIdx.x; i < total; i += kListThreads) out[i] = stage[i];
 }
 
+// First entry of every plane in the lists of the jobs that ask for it
+// (blockIdx.y: the job), from the entries' planes: entry i starts every
+// plane after entry i - 1's up to its own.
+__global__ void plane_starts_kernel(const ListJob* __restrict__ jobs) {
+  const ListJob& J = jobs[blockIdx.y];
+  if (!J.pstart) return;
+  const Geom& g = J.g;
+  const uint32_t n = *J.count;
+  auto plane = [&](uint32_t i) { return g.div_sz((J.list[i] & kListAt) - (uint32_t)g.off0); };
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i <= n; i += gridDim.x * blockDim.x) {
+    const int prev = i ? plane(i - 1) : -1, cur = i < n ? plane(i) : g.nz;
+    for (int k = prev + 1; k <= cur; ++k) J.pstart[k] = i;
+  }
+}
+
 // Many device buffers zeroed in one launch: blockIdx.y selects the buffer.
 __global__ void zero_many_kernel(const ZeroJob* __restrict__ jobs) {
   const ZeroJob J = jobs[blockIdx.y];
@@ -553,10 +568,11 @@ cudaError_t launch_coarse_coeffs(const LevelDev& Lc, unsigned long long* counts2
 cudaError_t launch_build_lists(const ListJob* jobs, int njobs, unsigned total_blocks, uint32_t* scratch,
                                cudaStream_t s) {
   if (njobs <= 0) return cudaSuccess;
-  count_launch(3);
+  count_launch(4);
   list_count_all_kernel<<<total_blocks, kListThreads, 0, s>>>(jobs, njobs, scratch);
   list_scan_all_kernel<<<njobs, 1024, 0, s>>>(jobs, scratch);
   list_write_all_kernel<<<total_blocks, kListThreads, 0, s>>>(jobs, njobs, scratch);
+  plane_starts_kernel<<<dim3(64, njobs), kListThreads, 0, s>>>(jobs);
   return cudaGetLastError();
 }
 

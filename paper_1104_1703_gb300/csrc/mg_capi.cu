@@ -334,6 +334,11 @@ mg_status iteration(mg_hierarchy* H, int l, int order, int prec = kFP64, bool up
   const void* cmat = (H->cmat_ok[order] && H->cmat_prec == prec) ? H->cmat[order] : nullptr;
   // the small coarse levels run as one single-CTA launch, which carries
   // the N_cycles recursion below level l itself
+  if (l >= 1 && l == H->cl_plan[order].first && !o.coarse_cluster)
+    return launch_ok(H, launch_cluster_cycle(H->L, H->cl_plan[order], order, o.n_pre, o.n_post, o.coarse_sweeps,
+                                             o.n_cycles, prec, H->cl_blobs[order], cmat, H->cmat_n[order],
+                                             H->err_flag + 3, H->cur),
+                     "coarse levels");
   if (l >= 1 && small_level(H->L[l].g))
     return launch_ok(H, launch_bottom(H->L, l, H->deepest[order], order, o.n_pre, o.n_post, o.coarse_sweeps,
                                       o.n_cycles, prec, cmat, H->cmat_n[order], H->cur),
@@ -404,13 +409,15 @@ mg_status norm2(mg_hierarchy* H, bool red_only, bool with_phi, double* out) {
   return MG_OK;
 }
 
-unsigned long long lists_hash(const mg_hierarchy* H) {
-  unsigned long long x = 1469598103934665603ULL;  // FNV-1a over every list length
-  for (int l = 0; l < H->nlev; ++l)
-    for (int i = 0; i < 6; ++i) {
-      x ^= H->L[l].hcount[i];
-      x *= 1099511628211ULL;
-    }
+// FNV-1a over what a mask build told the host: every list length and plane
+// start (the grids and shared-memory plans of a captured graph).
+unsigned long long build_hash(const mg_hierarchy* H) {
+  unsigned long long x = 1469598103934665603ULL;
+  const uint32_t* w = (const uint32_t*)H->hbuild_info;
+  for (size_t i = 0; i < H->build_info_bytes / sizeof(uint32_t); ++i) {
+    x ^= w[i];
+    x *= 1099511628211ULL;
+  }
   return x;
 }
 
@@ -478,7 +485,7 @@ mg_status capture_cycle(mg_hierarchy* H, int order, GraphSlot& gs) {
   if (st != MG_OK) return st;
   if (e != cudaSuccess || !gs.exec) return cuda_fail(H, e, "graph capture");
   gs.deepest = H->deepest[order];
-  gs.lists_hash = lists_hash(H);
+  gs.lists_hash = H->lists_hash;
   gs.nodes = t_captured;
   return MG_OK;
 }
@@ -502,7 +509,7 @@ mg_status run_cycle(mg_hierarchy* H, int order, double* r_out) {
     CKS(emit_cycle(H, order));
   } else {
     GraphSlot& gs = H->graphs[order][H->timing ? 1 : 0];
-    if (!gs.exec || gs.deepest != H->deepest[order] || gs.lists_hash != lists_hash(H))
+    if (!gs.exec || gs.deepest != H->deepest[order] || gs.lists_hash != H->lists_hash)
       CKS(capture_cycle(H, order, gs));
     CK(H, cudaGraphLaunch(gs.exec, H->stream));
     count_launch(gs.nodes);
@@ -520,6 +527,14 @@ mg_status run_cycle(mg_hierarchy* H, int order, double* r_out) {
     }
   }
   *r_out = std::sqrt(H->hscal[0]) / (H->h * H->h);
+  if (!std::isfinite(*r_out)) {  // a coarse-level launch whose wait ran out leaves NaN and its flag
+    int err = 0;
+    CK(H, cudaMemcpy(&err, H->err_flag + 3, sizeof(int), cudaMemcpyDeviceToHost));
+    if (err) {
+      CK(H, cudaMemset(H->err_flag + 3, 0, sizeof(int)));
+      return fail(H, MG_ERR_INTERNAL, "coarse levels: a neighbour's data did not arrive in time");
+    }
+  }
   if (H->opt.use_graphs && H->timing) {
     for (auto& p : H->graphs[order][1].events) {
       float ms = 0;
@@ -579,11 +594,12 @@ mg_status build_levels(mg_hierarchy* H, bool fine_built = false, const int8_t* m
   if (H->pass_on)
     CKS(launch_ok(H, launch_pass_tiles(H->L[0].g, H->L[0].code, H->pass_flags, H->pass_tiles, H->pass_ntiles, s),
                   "pass tiles"));
-  unsigned long long hc[2 * kMaxLevels];
-  CK(H, cudaMemcpyAsync(hc, H->counts, sizeof(hc), cudaMemcpyDeviceToHost, s));
-  for (int l = 0; l < H->nlev; ++l)
-    CK(H, cudaMemcpyAsync(H->L[l].hcount, H->L[l].count, sizeof(H->L[l].hcount), cudaMemcpyDeviceToHost, s));
+  CK(H, cudaMemcpyAsync((void*)H->hbuild_info, H->build_info, H->build_info_bytes, cudaMemcpyDeviceToHost, s));
   CK(H, cudaStreamSynchronize(s));
+  const unsigned long long* hc = (const unsigned long long*)H->hbuild_info;
+  for (int l = 0; l < H->nlev; ++l)
+    std::memcpy(H->L[l].hcount, H->hbuild_info + ((char*)H->L[l].count - H->build_info), sizeof(H->L[l].hcount));
+  H->lists_hash = build_hash(H);
   for (int c = 0; c < 2; ++c) H->L[0].hcount[2 + c] = H->L[0].hcount[4 + c];  // level 0: one active set
   for (int l = 0; l < H->nlev; ++l) {
     H->active[2][l] = (long long)hc[2 * l];
@@ -592,6 +608,16 @@ mg_status build_levels(mg_hierarchy* H, bool fine_built = false, const int8_t* m
   for (int o = 1; o <= 2; ++o) {
     H->deepest[o] = -1;
     for (int l = 0; l < H->nlev && H->active[o][l] > 0; ++l) H->deepest[o] = l;
+  }
+  // the coarse levels that run as one cluster launch (its residuals take the
+  // place of the red correction, which needs sweeps on both sides)
+  const int prec = H->opt.precision == 1 ? kFP32 : kFP64;
+  for (int o = 1; o <= 2; ++o) {
+    H->cl_plan[o] = ClPlan();
+    if (!H->cluster_ok || H->opt.n_pre < 1 || H->opt.n_post < 1) continue;
+    H->cl_plan[o] = cluster_plan(H->L, H->deepest[o], o, prec, H->cl_bound);
+    if (H->cl_plan[o].first)
+      CKS(launch_ok(H, launch_cluster_build(H->L, H->cl_plan[o], o, prec, H->cl_blobs[o], s), "coarse-level records"));
   }
   // the coarsest solve's map of each order, for the bottom cycle (one launch)
   const LevelDev* mapped[3] = {nullptr, nullptr, nullptr};
@@ -768,6 +794,7 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
   H->cur = H->stream;
   {
     cudaError_t e0 = init_cycle_kernels();
+    if (e0 == cudaSuccess) e0 = init_cluster_kernels(&H->cluster_ok);
     if (e0 != cudaSuccess) {
       mg_status st = cuda_fail(nullptr, e0, "kernel attributes");
       destroy(H);
@@ -784,7 +811,8 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
   // one arena for every level array
   Arena A;
   struct Off {
-    size_t phi[2], rhs[2], invd[2], diag[2], code[2], list[3][2], count, S;
+    size_t phi[2], rhs[2], invd[2], diag[2], code[2], list[3][2], S;
+    size_t pstart[3][2];  // in the build information
     size_t f_phi[2], f_rhs[2], f_invd[2], f_diag[2];
   } off[kMaxLevels];
   const bool mixed = o.precision == 1;
@@ -816,8 +844,19 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
       }
     }
     if (l > 0) off[l].S = A.reserve(sizeof(int32_t) * g.ncells());
-    off[l].count = A.reserve(sizeof(uint32_t) * 6);
   }
+  // build information: counts, list counts, plane starts
+  size_t info = sizeof(unsigned long long) * 2 * kMaxLevels + sizeof(uint32_t) * 6 * H->nlev;
+  for (int l = 1; l < H->nlev; ++l)
+    for (int ord = 1; ord <= 2; ++ord)
+      for (int c = 0; c < 2; ++c) {
+        off[l].pstart[ord][c] = info;
+        if (cluster_level(H->L[l].g)) info += sizeof(uint32_t) * (H->L[l].g.nz + 1);
+      }
+  const size_t o_info = A.reserve(info);
+  H->cl_bound = H->cluster_ok ? cluster_blob_bound(H->L, H->nlev, mixed ? kFP32 : kFP64) : 0;
+  size_t o_blobs[3] = {0, 0, 0};
+  for (int ord = 1; ord <= 2; ++ord) o_blobs[ord] = A.reserve(H->cl_bound);
   // batched build launches: one scratch word per list block of every list
   std::vector<ListJob> ljobs;
   unsigned lblocks = 0;
@@ -872,7 +911,6 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
   const int cprec = mixed ? kFP32 : kFP64;
   size_t o_cmat[3] = {0, 0, 0};
   for (int ord = 1; ord <= 2 && cmaps; ++ord) o_cmat[ord] = A.reserve(coarse_map_bytes(cprec));
-  size_t o_cnt = A.reserve(sizeof(unsigned long long) * 2 * kMaxLevels);
 
   cudaError_t e = dev_malloc((void**)&H->arena, A.used);
   if (e != cudaSuccess) {
@@ -881,7 +919,7 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
     destroy(H);
     return st;
   }
-  e = host_malloc((void**)&H->hscal, sizeof(double) * 8);
+  e = host_malloc((void**)&H->hscal, sizeof(double) * 8 + info);  // scalars, then the build information
   if (e != cudaSuccess) {
     H->hscal = nullptr;
     mg_status st = cuda_fail(nullptr, e, "cudaMallocHost");
@@ -889,6 +927,10 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
     return st;
   }
   char* base = H->arena;
+  for (int ord = 1; ord <= 2; ++ord) H->cl_blobs[ord] = base + o_blobs[ord];
+  H->build_info = base + o_info;
+  H->build_info_bytes = info;
+  H->hbuild_info = (const char*)(H->hscal + 8);
   for (int l = 0; l < H->nlev; ++l) {
     for (int c = 0; c < 2; ++c) {
       H->L[l].phi[c] = (double*)(base + off[l].phi[c]);
@@ -906,7 +948,13 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
       H->L[l].diag[c] = l > 0 ? (double*)(base + off[l].diag[c]) : nullptr;
     }
     H->L[l].S = l > 0 ? (int32_t*)(base + off[l].S) : nullptr;
-    H->L[l].count = (uint32_t*)(base + off[l].count);
+    H->L[l].count = (uint32_t*)(H->build_info + sizeof(unsigned long long) * 2 * kMaxLevels) + 6 * l;
+    if (l > 0 && cluster_level(H->L[l].g))
+      for (int ord = 1; ord <= 2; ++ord)
+        for (int c = 0; c < 2; ++c) {
+          H->L[l].pstart[ord][c] = (uint32_t*)(H->build_info + off[l].pstart[ord][c]);
+          H->L[l].hpstart[ord][c] = (const uint32_t*)(H->hbuild_info + off[l].pstart[ord][c]);
+        }
   }
   H->list_scratch = (uint32_t*)(base + o_lscr);
   H->list_jobs = (ListJob*)(base + o_ljobs);
@@ -932,7 +980,7 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
   H->cmat_prec = cprec;
   for (int ord = 1; ord <= 2; ++ord) H->cmat[ord] = cmaps ? (void*)(base + o_cmat[ord]) : nullptr;
   for (int l = 0; l < H->nlev; ++l) H->L[l].g.fault = (unsigned*)(H->err_flag + 1);
-  H->counts = (unsigned long long*)(base + o_cnt);
+  H->counts = (unsigned long long*)H->build_info;
   if (pass) {
     for (int c = 0; c < 2; ++c) H->phi32_alt[c] = (float*)(base + o_alt[c]);
     H->pass_flags = (uint32_t*)(base + o_pflags);
@@ -962,6 +1010,7 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
           ljobs[jn].code = H->L[l].code[c];
           ljobs[jn].list = H->L[l].list[o][c];
           ljobs[jn].count = H->L[l].count + o * 2 + c;
+          ljobs[jn].pstart = o > 0 ? H->L[l].pstart[o][c] : nullptr;
         }
     std::vector<ZeroJob> zjobs;
     for (int l = 0; l < H->nlev; ++l)

@@ -107,6 +107,11 @@ struct LevelDev {
   uint32_t* list[3][2];
   uint32_t* count;
   uint32_t hcount[6];  // host copy of count (sizes the launch grids)
+  // Levels the cluster cycle may take (cluster_level): pstart[order][colour][k]
+  // is the first entry of plane k in that list (nz + 1 entries; device memory)
+  // and hpstart the host's copy; nullptr elsewhere.
+  uint32_t* pstart[3][2] = {};
+  const uint32_t* hpstart[3][2] = {};
   double* rhsd[2];     // level 0 of the FP64 method: b / D (nullptr elsewhere)
   int exact_sum = 0;   // level 0: FP64 neighbour sums in integer arithmetic (exact_sum.cuh)
   int seg_shift = 0;   // level 0: log2 of the row-segment length (0: no segment lists)
@@ -178,6 +183,7 @@ struct ListJob {
   int colour;
   uint8_t bit;
   int seg_shift;
+  uint32_t* pstart;  // nullable: the list's plane starts (LevelDev), written after the list
 };
 // list entries a job scans (cells, or row segments with seg_shift > 0)
 __host__ __device__ inline long long list_job_slots(const Geom& g, int seg_shift) {
