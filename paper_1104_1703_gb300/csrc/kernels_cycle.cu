@@ -1204,13 +1204,19 @@ __global__ void __launch_bounds__(kMidThreads, 1) mid_kernel(MidArgs<T> a) {
 // is the result (x_r, x_b) of `sweeps` red-black sweeps of the deepest level
 // started from a unit input, b = e_j for j < n_r + n_b with a zero initial
 // correction, or the initial black correction e_(j - n_r - n_b) with b = 0.
-// One warp per column, kCmWarps columns per CTA.  Each CTA first indexes the
+// One warp per column, CmWarps columns per CTA (FP64: one warp per
+// scheduler, each of which takes 64 cycles per FP64 warp instruction; with 16
+// warps per CTA the 100 dependent half-sweeps took 81 us instead of 37 on a
+// 4^3 level, while other SMs idled).  Each CTA first indexes the
 // level's unknowns: slot -> position in its colour's list, then per unknown
 // the positions of its six neighbours of the other colour (-1 for a slot
 // that is not an unknown: it holds 0).  The sweeps then run on the unknowns'
 // values alone, in per-warp shared-memory vectors, with the operator's own
 // arithmetic and summation order: (sum of the six neighbours - b) * (1/D).
-constexpr int kCmWarps = 16;
+template <typename T>
+struct CmWarps {
+  static constexpr int value = sizeof(T) == 8 ? 4 : 16;
+};
 constexpr long long kCmMaxSlots = 8192;  // slots per colour array of a level the map is built for
 
 template <typename T>
@@ -1228,7 +1234,7 @@ struct CoarseMatSmem {
   int8_t map[2][kCmMaxSlots];
   int8_t nbr[2][kCoarseMatMax][6];
   T id[2][kCoarseMatMax];
-  T xs[kCmWarps][2][kCoarseMatMax];
+  T xs[CmWarps<T>::value][2][kCoarseMatMax];
 };
 
 template <int KIND, typename T>
@@ -1240,7 +1246,7 @@ __device__ void coarse_matrix_body(const CoarseMatArgs<T>& a, CoarseMatSmem<T>& 
   const Geom& g = a.g;
   const uint32_t nr = a.n[0], nb = a.n[1], nt = nr + nb, ncol = nt + nb;
   if (g.total > kCmMaxSlots || nt > (uint32_t)kCoarseMatMax) return;
-  if (blockIdx.x * kCmWarps >= ncol) return;  // the other order's map needs more CTAs
+  if (blockIdx.x * CmWarps<T>::value >= ncol) return;  // the other order's map needs more CTAs
   for (long long e = threadIdx.x; e < 2 * g.total; e += blockDim.x) map[e >= g.total][e % g.total] = -1;
   __syncthreads();
   for (uint32_t e = threadIdx.x; e < nt; e += blockDim.x) {
@@ -1263,7 +1269,7 @@ __device__ void coarse_matrix_body(const CoarseMatArgs<T>& a, CoarseMatSmem<T>& 
   }
   __syncthreads();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t j = blockIdx.x * kCmWarps + w;
+  const uint32_t j = blockIdx.x * CmWarps<T>::value + w;
   if (j >= ncol) return;
   T(*x)[kCoarseMatMax] = xs[w];
   for (uint32_t u = lane; u < (uint32_t)kCoarseMatMax; u += 32) {
@@ -1291,7 +1297,7 @@ __device__ void coarse_matrix_body(const CoarseMatArgs<T>& a, CoarseMatSmem<T>& 
 // first-order operator, D = 6), 1 order 2's; an order with no map has no
 // columns.
 template <typename T>
-__global__ void __launch_bounds__(kCmWarps * 32) coarse_matrix_kernel(CoarseMatArgs<T> a1, CoarseMatArgs<T> a2) {
+__global__ void __launch_bounds__(CmWarps<T>::value * 32) coarse_matrix_kernel(CoarseMatArgs<T> a1, CoarseMatArgs<T> a2) {
   __shared__ CoarseMatSmem<T> sm;
   if (blockIdx.y == 0) coarse_matrix_body<2, T>(a1, sm);
   else coarse_matrix_body<1, T>(a2, sm);
@@ -1525,10 +1531,10 @@ template <typename T>
 cudaError_t coarse_maps_t(const LevelDev* L1, const LevelDev* L2, int sweeps, T* out1, T* out2, cudaStream_t s) {
   const CoarseMatArgs<T> a1 = coarse_map_args(L1, 1, sweeps, out1), a2 = coarse_map_args(L2, 2, sweeps, out2);
   const uint32_t n1 = a1.n[0] + 2 * a1.n[1], n2 = a2.n[0] + 2 * a2.n[1];
-  const unsigned grid = ((n1 > n2 ? n1 : n2) + kCmWarps - 1) / kCmWarps;
+  const unsigned grid = ((n1 > n2 ? n1 : n2) + CmWarps<T>::value - 1) / CmWarps<T>::value;
   if (grid == 0) return cudaSuccess;
   count_launch();
-  coarse_matrix_kernel<T><<<dim3(grid, 2), kCmWarps * 32, 0, s>>>(a1, a2);
+  coarse_matrix_kernel<T><<<dim3(grid, 2), CmWarps<T>::value * 32, 0, s>>>(a1, a2);
   return cudaGetLastError();
 }
 
