@@ -21,6 +21,7 @@
 #include <cmath>
 
 #include "../../include/mg.h"
+#include "exact_sum.cuh"
 #include "mg_internal.h"
 
 namespace gbmg {
@@ -38,51 +39,92 @@ constexpr int kNoAllocThreads = 256;
 // the first kernel of the same call, so nothing needs clearing between calls.
 static __device__ __align__(256) double g_noalloc_partials[kNoAllocMaxPartials];
 
+// 2 x in integer arithmetic (a zero or subnormal x gives 0, as exact_sum takes it).
+__device__ __forceinline__ double twice(double x) {
+  const unsigned long long b = bits_of(x);
+  const unsigned e = (unsigned)(b >> 52) & 0x7ffu;
+  if (e == 0) return 0.0;
+  if (e == 0x7ffu) return x;
+  if (e == 0x7feu) return double_of((b & 0x8000000000000000ull) | 0x7ff0000000000000ull);
+  return double_of(b + (1ull << 52));
+}
+
 // Residual r^ = h^2 (Laplacian Phi - rho) of every active cell, with the
 // modified stencil of Section 3 at level 0 (ghost at theta = 1/2 through the
 // face value Phi_b, Fig. 5): r^ = sum_active Phi_j + 2 sum_ghost Phi_b
 // - (6 + #ghost) Phi_i - h^2 rho_i.  Block sums of r^2 go to partials.
+//
+// A thread per cell ran about 12 FP64 operations for active and idle lanes
+// alike, on a pipe that takes 16 cycles per warp instruction (504 us on a
+// half-active 256^3 patch with face values, whose 688 MB take 102 us).  So a
+// warp takes kTile cells of a row, lists the active ones and works with every
+// lane in use, and the six terms are added in integer arithmetic
+// (exact_sum.cuh), which leaves three FP64 instructions per active cell.
+constexpr int kTile = 128;
+
 __global__ void __launch_bounds__(kNoAllocThreads)
 noalloc_resnorm_kernel(const int8_t* __restrict__ mask, const double* __restrict__ phi,
                        const double* __restrict__ rho, const double* __restrict__ bx,
                        const double* __restrict__ by, const double* __restrict__ bz, int nx, int ny, int nz,
                        double h2, double* partials) {
-  const long long n = (long long)nx * ny * nz;
+  constexpr int kWarps = kNoAllocThreads / 32;
+  __shared__ uint8_t active[kWarps][kTile];
+  __shared__ double diag[8];  // 6 + #ghost
+  if (threadIdx.x < 8) diag[threadIdx.x] = (double)(6 + (int)threadIdx.x);
+  __syncthreads();
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long sy = nx, sz = (long long)nx * ny;
+  const unsigned tiles = (unsigned)(nx + kTile - 1) / kTile;
+  const unsigned n = tiles * (unsigned)ny * (unsigned)nz;
   double acc = 0.0;
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
-       idx += (long long)gridDim.x * blockDim.x) {
-    if (mask[idx] <= 0) continue;
-    const int i = (int)(idx % nx);
-    const long long t = idx / nx;
-    const int j = (int)(t % ny), k = (int)(t / ny);
-    const long long fx = ((long long)k * ny + j) * (nx + 1) + i;
-    const long long fy = ((long long)k * (ny + 1) + j) * nx + i;
-    const long long fz = idx;
-    const bool in[6] = {i > 0, i + 1 < nx, j > 0, j + 1 < ny, k > 0, k + 1 < nz};
-    const long long off[6] = {-1, 1, -sy, sy, -sz, sz};
-    const double* fb[6] = {bx, bx, by, by, bz, bz};
-    const long long fi[6] = {fx, fx + 1, fy, fy + nx, fz, fz + sz};
-    double s = 0.0;
-    int ghosts = 0;
+  for (unsigned t = blockIdx.x * kWarps + w; t < n; t += gridDim.x * kWarps) {
+    const unsigned row = t / tiles;
+    const int k = (int)(row / (unsigned)ny), j = (int)(row - (unsigned)k * (unsigned)ny);
+    const int i0 = (int)(t - row * tiles) * kTile;
+    const long long r0 = (long long)row * nx;  // cell (0, j, k)
+    const int8_t* __restrict__ m = mask + r0;
+    int na = 0;
 #pragma unroll
-    for (int d = 0; d < 6; ++d) {
-      if (in[d] && mask[idx + off[d]] > 0) {
-        s += phi[idx + off[d]];
-      } else {
-        ++ghosts;
-        if (fb[d]) s += 2.0 * fb[d][fi[d]];
-      }
+    for (int s = 0; s < kTile / 32; ++s) {
+      const int i = i0 + 32 * s + lane;
+      const bool act = i < nx && m[i] > 0;
+      const unsigned all = __ballot_sync(0xffffffffu, act);
+      if (act) active[w][na + __popc(all & ((1u << lane) - 1u))] = (uint8_t)(32 * s + lane);
+      na += __popc(all);
     }
-    const double r = fma(-(double)(6 + ghosts), phi[idx], s) - h2 * rho[idx];
-    acc = fma(r, r, acc);
+    __syncwarp();
+    const bool row_in[4] = {j > 0, j + 1 < ny, k > 0, k + 1 < nz};
+    const double* __restrict__ fx = bx ? bx + (long long)row * (nx + 1) : nullptr;
+    const double* __restrict__ fy = by ? by + ((long long)k * (ny + 1) + j) * nx : nullptr;
+    const double* __restrict__ fz = bz ? bz + r0 : nullptr;
+    const double* __restrict__ p = phi + r0;
+    for (int x = lane; x < na; x += 32) {
+      const int i = i0 + active[w][x];
+      const bool in[6] = {i > 0 && m[i - 1] > 0,         i + 1 < nx && m[i + 1] > 0,    row_in[0] && m[i - sy] > 0,
+                          row_in[1] && m[i + sy] > 0,    row_in[2] && m[i - sz] > 0,    row_in[3] && m[i + sz] > 0};
+      const long long off[6] = {-1, 1, -sy, sy, -sz, sz};
+      const double* f[6] = {fx ? fx + i : nullptr, fx ? fx + i + 1 : nullptr, fy ? fy + i : nullptr,
+                            fy ? fy + i + nx : nullptr, fz ? fz + i : nullptr, fz ? fz + i + sz : nullptr};
+      double v[6];
+      int ghosts = 0;
+#pragma unroll
+      for (int d = 0; d < 6; ++d) {
+        v[d] = 0.0;
+        if (in[d]) v[d] = p[i + off[d]];
+        else if (f[d]) v[d] = twice(*f[d]);
+        ghosts += !in[d];
+      }
+      const double r = fma(-diag[ghosts], p[i], exact_sum(v)) - h2 * rho[r0 + i];
+      acc = fma(r, r, acc);
+    }
+    __syncwarp();
   }
-  __shared__ double warp_sums[kNoAllocThreads / 32];
+  __shared__ double warp_sums[kWarps];
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) warp_sums[threadIdx.x >> 5] = acc;
+  if (lane == 0) warp_sums[w] = acc;
   __syncthreads();
   if (threadIdx.x < 32) {
-    double v = threadIdx.x < kNoAllocThreads / 32 ? warp_sums[threadIdx.x] : 0.0;
+    double v = threadIdx.x < kWarps ? warp_sums[threadIdx.x] : 0.0;
     for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
     if (threadIdx.x == 0) partials[blockIdx.x] = v;
   }
@@ -140,8 +182,10 @@ extern "C" mg_status mg_residual_norm_noalloc(const int8_t* mask, const double* 
     set_thread_error("mg_residual_norm_noalloc: cudaGetSymbolAddress of the scratch array failed");
     return MG_ERR_CUDA;
   }
-  const long long n = (long long)nx * ny * nz;
-  long long blocks = (n + kNoAllocThreads - 1) / kNoAllocThreads;
+  // a warp per tile of a row, at most 8 resident blocks per multiprocessor
+  const long long tiles = (long long)((nx + kTile - 1) / kTile) * ny * nz;
+  long long blocks = (tiles + kNoAllocThreads / 32 - 1) / (kNoAllocThreads / 32);
+  if (blocks > 8LL * device_sms()) blocks = 8LL * device_sms();
   if (blocks > kNoAllocMaxPartials) blocks = kNoAllocMaxPartials;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const double h2 = h * h;
