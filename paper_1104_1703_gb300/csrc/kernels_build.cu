@@ -257,57 +257,126 @@ __global__ void fold_faces_kernel(LevelDev L, FineExtra F, const double* __restr
   }
 }
 
-// Trilinear interpolation of the coarse AMR potential at a point given in
-// fine-cell units; coarse cell (I,J,K) is centred at o + 2I + 1.
+// Trilinear interpolation of the coarse AMR potential at a face centre given
+// in half fine cells (x2, y2, z2: twice the position); coarse cell (I,J,K) is
+// centred at o + 2I + 1 fine cells.  Along an axis the position in coarse
+// cells from the first centre is (x2 - 2 o - 2) / 4: its integer part and the
+// quarters of its fraction are exact in integers, so the weights cost no FP64
+// instruction.
 __device__ __forceinline__ bool coarse_sample(const double* __restrict__ pc, int cnx, int cny, int cnz, int ox,
-                                              int oy, int oz, double px, double py, double pz, double& out) {
-  const double u = (px - ox) * 0.5 - 0.5, v = (py - oy) * 0.5 - 0.5, w = (pz - oz) * 0.5 - 0.5;
-  const double fu = floor(u), fv = floor(v), fw = floor(w);
-  const int I = (int)fu, J = (int)fv, K = (int)fw;
+                                              int oy, int oz, int x2, int y2, int z2, double& out) {
+  const int qx = x2 - 2 * ox - 2, qy = y2 - 2 * oy - 2, qz = z2 - 2 * oz - 2;
+  const int I = qx >> 2, J = qy >> 2, K = qz >> 2;
   if (I < 0 || J < 0 || K < 0 || I + 1 >= cnx || J + 1 >= cny || K + 1 >= cnz) return false;
-  const double tu = u - fu, tv = v - fv, tw = w - fw;
+  // quarters 0 .. 3 as doubles: 0, 0x3fd00000'00000000, 0x3fe.., 0x3fe8..
+  auto quarters = [](int q) {
+    return __hiloint2double(q == 0 ? 0 : (q == 1 ? 0x3fd00000 : (q == 2 ? 0x3fe00000 : 0x3fe80000)), 0);
+  };
+  const double tu = quarters(qx & 3), tv = quarters(qy & 3), tw = quarters(qz & 3);
+  // 1 - t exactly (q = 0 gives 1)
+  auto rest = [&](int q) { return q == 0 ? __hiloint2double(0x3ff00000, 0) : quarters(4 - q); };
+  const double su = rest(qx & 3), sv = rest(qy & 3), sw = rest(qz & 3);
   const long long sy = cnx, sz = (long long)cnx * cny;
   const double* p = pc + K * sz + (long long)J * sy + I;
-  const double c00 = (1.0 - tu) * p[0] + tu * p[1];
-  const double c10 = (1.0 - tu) * p[sy] + tu * p[sy + 1];
-  const double c01 = (1.0 - tu) * p[sz] + tu * p[sz + 1];
-  const double c11 = (1.0 - tu) * p[sz + sy] + tu * p[sz + sy + 1];
-  const double c0 = (1.0 - tv) * c00 + tv * c10;
-  const double c1 = (1.0 - tv) * c01 + tv * c11;
-  out = (1.0 - tw) * c0 + tw * c1;
+  const double c00 = su * p[0] + tu * p[1];
+  const double c10 = su * p[sy] + tu * p[sy + 1];
+  const double c01 = su * p[sz] + tu * p[sz + 1];
+  const double c11 = su * p[sz + sy] + tu * p[sz + sy + 1];
+  const double c0 = sv * c00 + tv * c10;
+  const double c1 = sv * c01 + tv * c11;
+  out = sw * c0 + tw * c1;
   return true;
 }
 
+// Twice the centre of face d (-x, +x, -y, +y, -z, +z) of cell (i, j, k).
+__device__ __forceinline__ void face_centre2(int d, int i, int j, int k, int& x2, int& y2, int& z2) {
+  const int a = d >> 1, s = (d & 1) ? 1 : -1;
+  x2 = 2 * i + 1 + (a == 0 ? s : 0);
+  y2 = 2 * j + 1 + (a == 1 ? s : 0);
+  z2 = 2 * k + 1 + (a == 2 ? s : 0);
+}
+
 // K7 + K3: Dirichlet values interpolated from the coarser AMR level at the
-// centre of each ghost face, folded into bc.
-__global__ void fold_coarse_kernel(LevelDev L, FineExtra F, const double* __restrict__ pc, int cnx, int cny,
-                                   int cnz, int ox, int oy, int oz, int* err_flag) {
+// centre of each ghost face, folded into bc, and b = h^2 rho - bc in the same
+// pass.
+//
+// Only the FP64 pipe (2 lanes per clock and SM, idle lanes included) bounds
+// it: about 17 operations per face, and a thread per cell ran them for every
+// direction in every warp (320 us on a half-active 128^3 blob patch).  So a
+// warp takes 128 cells of a row at a time, lists their ghost faces and their
+// boundary cells, and works through both lists with every lane in use; the
+// other cells only copy h^2 rho.
+constexpr int kFoldWarps = 4;
+constexpr int kFoldCells = 128;
+
+__global__ void __launch_bounds__(32 * kFoldWarps)
+    fold_coarse_kernel(LevelDev L, FineExtra F, const double* __restrict__ pc, int cnx, int cny, int cnz, int ox,
+                       int oy, int oz, int* err_flag) {
+  __shared__ double vals[kFoldWarps][6 * kFoldCells];
+  __shared__ uint16_t faces[kFoldWarps][6 * kFoldCells];     // cell | direction << 8
+  __shared__ uint16_t cells[kFoldWarps][kFoldCells];         // boundary cells of the tile
+  __shared__ uint16_t start[kFoldWarps][kFoldCells + 1];     // their first face
   const Geom g = L.g;
-  const long long n = g.ncells();
-  for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
-       idx += (long long)gridDim.x * blockDim.x) {
-    int i, j, k;
-    natural_coords(idx, g.nx, g.ny, i, j, k);
-    const int c = colour_of(i, j, k);
-    const long long at = g.at(i >> 1, j, k);
-    const uint8_t code = L.code[c][at];
-    double acc = 0.0;
-    if (code & kActive2) {
-      const int gh = code >> kGhostShift;
-      const double x = i + 0.5, y = j + 0.5, z = k + 0.5;
-      const double fx[6] = {(double)i, (double)(i + 1), x, x, x, x};
-      const double fy[6] = {y, y, (double)j, (double)(j + 1), y, y};
-      const double fz[6] = {z, z, z, z, (double)k, (double)(k + 1)};
-      for (int d = 0; d < 6; ++d) {
-        if (!(gh & (1 << d))) continue;
-        double v;
-        if (coarse_sample(pc, cnx, cny, cnz, ox, oy, oz, fx[d], fy[d], fz[d], v))
-          acc += v;
-        else
-          atomicExch(err_flag, 1);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned tiles = (unsigned)(g.nx + kFoldCells - 1) / kFoldCells;
+  const unsigned n = tiles * (unsigned)g.ny * (unsigned)g.nz;
+  for (unsigned t = blockIdx.x * kFoldWarps + w; t < n; t += gridDim.x * kFoldWarps) {
+    const unsigned row = t / tiles;
+    const int k = (int)(row / (unsigned)g.ny), j = (int)(row - (unsigned)k * (unsigned)g.ny);
+    const int i0 = (int)(t - row * tiles) * kFoldCells;
+    const long long base = g.at(0, j, k);
+    int nf = 0, nc = 0;
+#pragma unroll
+    for (int s = 0; s < kFoldCells / 32; ++s) {
+      const int i = i0 + 32 * s + lane;
+      const bool in = i < g.nx;
+      const int c = colour_of(i, j, k);
+      const long long at = base + (i >> 1);
+      const uint8_t code = in ? L.code[c][at] : 0;
+      const int gh = (code & kActive2) ? code >> kGhostShift : 0;
+      const int cnt = __popc(gh);
+      const unsigned have = __ballot_sync(0xffffffffu, cnt > 0);
+      int incl = cnt;
+      for (int off = 1; off < 32; off <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += v;
       }
+      if (cnt) {
+        const int rank = nc + __popc(have & ((1u << lane) - 1u));
+        int pos = nf + incl - cnt;
+        cells[w][rank] = (uint16_t)(32 * s + lane);
+        start[w][rank] = (uint16_t)pos;
+        for (int d = 0; d < 6; ++d)
+          if (gh & (1 << d)) faces[w][pos++] = (uint16_t)((32 * s + lane) | (d << 8));
+      } else if (in) {
+        (c ? F.bc[1] : F.bc[0])[at] = 0.0;
+        (c ? L.rhs[1] : L.rhs[0])[at] = (c ? F.rhoh2[1] : F.rhoh2[0])[at];
+      }
+      nc += __popc(have);
+      nf += __shfl_sync(0xffffffffu, incl, 31);
     }
-    F.bc[c][at] = 2.0 * acc;
+    if (lane == 0) start[w][nc] = (uint16_t)nf;
+    __syncwarp();
+    for (int x = lane; x < nf; x += 32) {
+      const int e = faces[w][x];
+      int x2, y2, z2;
+      face_centre2(e >> 8, i0 + (e & 255), j, k, x2, y2, z2);
+      double v = 0.0;
+      if (!coarse_sample(pc, cnx, cny, cnz, ox, oy, oz, x2, y2, z2, v)) atomicExch(err_flag, 1);
+      vals[w][x] = v;
+    }
+    __syncwarp();
+    for (int x = lane; x < nc; x += 32) {
+      const int i = i0 + cells[w][x];
+      const int c = colour_of(i, j, k);
+      const long long at = base + (i >> 1);
+      double acc = 0.0;
+      for (int f = start[w][x]; f < start[w][x + 1]; ++f) acc += vals[w][f];
+      const double bc = 2.0 * acc;
+      (c ? F.bc[1] : F.bc[0])[at] = bc;
+      (c ? L.rhs[1] : L.rhs[0])[at] = (c ? F.rhoh2[1] : F.rhoh2[0])[at] - bc;
+    }
+    __syncwarp();
   }
 }
 
@@ -329,18 +398,16 @@ __global__ void faces_from_coarse_kernel(LevelDev L, const double* __restrict__ 
     if (!(code & kActive2)) continue;
     const int gh = code >> kGhostShift;
     if (!gh) continue;
-    const double x = i + 0.5, y = j + 0.5, z = k + 0.5;
-    const double fx[6] = {(double)i, (double)(i + 1), x, x, x, x};
-    const double fy[6] = {y, y, (double)j, (double)(j + 1), y, y};
-    const double fz[6] = {z, z, z, z, (double)k, (double)(k + 1)};
     const long long nx1 = g.nx + 1, ny1 = g.ny + 1;
     double* const dst[6] = {bx + ((long long)k * g.ny + j) * nx1 + i, bx + ((long long)k * g.ny + j) * nx1 + i + 1,
                             by + ((long long)k * ny1 + j) * g.nx + i, by + ((long long)k * ny1 + j + 1) * g.nx + i,
                             bz + ((long long)k * g.ny + j) * g.nx + i, bz + ((long long)(k + 1) * g.ny + j) * g.nx + i};
     for (int d = 0; d < 6; ++d) {
       if (!(gh & (1 << d))) continue;
+      int x2, y2, z2;
+      face_centre2(d, i, j, k, x2, y2, z2);
       double v;
-      if (coarse_sample(pc, cnx, cny, cnz, ox, oy, oz, fx[d], fy[d], fz[d], v)) *dst[d] = v;
+      if (coarse_sample(pc, cnx, cny, cnz, ox, oy, oz, x2, y2, z2, v)) *dst[d] = v;
       else atomicExch(err_flag, 1);
     }
   }
@@ -535,6 +602,10 @@ __global__ void zero_many_kernel(const ZeroJob* __restrict__ jobs) {
     p[e] = 0ull;
 }
 
+// An origin outside +-2^28 puts every face outside the coarse centres, as its
+// clamped value does, whose doubled coordinates fit 32 bits.
+int clamp_origin(int o) { return o < -(1 << 28) ? -(1 << 28) : (o > (1 << 28) ? (1 << 28) : o); }
+
 int grid_for(long long n) {
   long long b = (n + kThreads - 1) / kThreads;
   if (b < 1) b = 1;
@@ -623,16 +694,19 @@ cudaError_t launch_fold_faces(const LevelDev& L0, const FineExtra& F, const doub
 cudaError_t launch_fold_coarse(const LevelDev& L0, const FineExtra& F, const double* pc, int cnx, int cny,
                                int cnz, int ox, int oy, int oz, int* err_flag, cudaStream_t s) {
   count_launch();
-  fold_coarse_kernel<<<grid_for(L0.g.ncells()), kThreads, 0, s>>>(L0, F, pc, cnx, cny, cnz, ox, oy, oz,
-                                                                   err_flag);
+  const long long tiles = (long long)((L0.g.nx + kFoldCells - 1) / kFoldCells) * L0.g.ny * L0.g.nz;
+  long long blocks = (tiles + kFoldWarps - 1) / kFoldWarps;
+  if (blocks > 32LL * device_sms()) blocks = 32LL * device_sms();
+  fold_coarse_kernel<<<(int)blocks, 32 * kFoldWarps, 0, s>>>(L0, F, pc, cnx, cny, cnz, clamp_origin(ox), clamp_origin(oy),
+                                                          clamp_origin(oz), err_flag);
   return cudaGetLastError();
 }
 
 cudaError_t launch_faces_from_coarse(const LevelDev& L0, const double* pc, int cnx, int cny, int cnz, int ox, int oy,
                                     int oz, double* bx, double* by, double* bz, int* err_flag, cudaStream_t s) {
   count_launch();
-  faces_from_coarse_kernel<<<grid_for(L0.g.ncells()), kThreads, 0, s>>>(L0, pc, cnx, cny, cnz, ox, oy, oz, bx, by, bz,
-                                                                         err_flag);
+  faces_from_coarse_kernel<<<grid_for(L0.g.ncells()), kThreads, 0, s>>>(
+      L0, pc, cnx, cny, cnz, clamp_origin(ox), clamp_origin(oy), clamp_origin(oz), bx, by, bz, err_flag);
   return cudaGetLastError();
 }
 

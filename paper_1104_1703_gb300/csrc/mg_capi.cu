@@ -697,6 +697,17 @@ mg_status check_faults(mg_hierarchy* H) {
 
 namespace {
 
+// True when every face centre of the box lies between the coarse cell centres
+// (coarse_sample's test at both ends of each axis; positions in between pass
+// when the ends do).
+bool coarse_covers(const Geom& g, int cnx, int cny, int cnz, int ox, int oy, int oz) {
+  auto axis = [](long long n, long long cn, long long o) {
+    const long long lo = -2 * o - 2, hi = 2 * n - 2 * o - 2;
+    return lo >= 0 && (hi >> 2) + 1 < cn;
+  };
+  return axis(g.nx, cnx, ox) && axis(g.ny, cny, oy) && axis(g.nz, cnz, oz);
+}
+
 mg_status check_level(mg_hierarchy* H, int level) {
   if (!H) return fail(H, MG_ERR_INVALID_ARG, "null hierarchy");
   if (level < 0 || level >= H->nlev) return fail(H, MG_ERR_INVALID_ARG, "level out of range");
@@ -1135,11 +1146,21 @@ mg_status mg_set_dirichlet_from_coarse(mg_hierarchy* H, const double* phi_c, mg_
   if (where == MG_MEM_HOST) CKS(ensure_staging(H, bytes));
   const void* src;
   CKS(device_view(H, phi_c, where, bytes, 0, &src));
-  CK(H, cudaMemsetAsync(H->err_flag, 0, sizeof(int), H->stream));
+  // a coarse grid that covers every face of the box needs no look at the
+  // flag, so the call does not wait
+  const bool covered = coarse_covers(H->L[0].g, cnx, cny, cnz, ox, oy, oz);
+  if (!covered) CK(H, cudaMemsetAsync(H->err_flag, 0, sizeof(int), H->stream));
   H->bc_zero = false;
+  H->r_zero_valid = false;
+  H->rhsd_valid = false;
+  H->prepared = false;
   CKS(launch_ok(H, launch_fold_coarse(H->L[0], H->F, (const double*)src, cnx, cny, cnz, ox, oy, oz, H->err_flag,
                                      H->stream),
                 "coarse interpolation"));
+  if (covered) {
+    if (where == MG_MEM_HOST) CK(H, cudaStreamSynchronize(H->stream));
+    return MG_OK;
+  }
   int err = 0;
   CK(H, cudaMemcpyAsync(H->hscal, H->err_flag, sizeof(int), cudaMemcpyDeviceToHost, H->stream));
   CK(H, cudaStreamSynchronize(H->stream));
@@ -1148,16 +1169,9 @@ mg_status mg_set_dirichlet_from_coarse(mg_hierarchy* H, const double* phi_c, mg_
     CKS(zero_split(H, H->L[0].g, H->F.bc));
     H->bc_zero = true;
     CKS(launch_ok(H, launch_combine_rhs(H->L[0], H->F, H->stream), "rhs fold"));
-    H->r_zero_valid = false;
-    H->rhsd_valid = false;
-  H->prepared = false;
     return fail(H, MG_ERR_INVALID_ARG,
                 "a boundary face lies outside the coarse cell centres; Dirichlet values reset to 0");
   }
-  CKS(launch_ok(H, launch_combine_rhs(H->L[0], H->F, H->stream), "rhs fold"));
-  H->r_zero_valid = false;
-  H->rhsd_valid = false;
-  H->prepared = false;
   return MG_OK;
 }
 
@@ -1178,10 +1192,15 @@ mg_status mg_faces_from_coarse(mg_hierarchy* H, const double* phi_c, mg_mem wher
   CK(H, cudaMemsetAsync(bx, 0, sizeof(double) * (size_t)(g.nx + 1) * g.ny * g.nz, H->stream));
   CK(H, cudaMemsetAsync(by, 0, sizeof(double) * (size_t)g.nx * (g.ny + 1) * g.nz, H->stream));
   CK(H, cudaMemsetAsync(bz, 0, sizeof(double) * (size_t)g.nx * g.ny * (g.nz + 1), H->stream));
-  CK(H, cudaMemsetAsync(H->err_flag, 0, sizeof(int), H->stream));
+  const bool covered = coarse_covers(g, cnx, cny, cnz, ox, oy, oz);
+  if (!covered) CK(H, cudaMemsetAsync(H->err_flag, 0, sizeof(int), H->stream));
   CKS(launch_ok(H, launch_faces_from_coarse(H->L[0], (const double*)src, cnx, cny, cnz, ox, oy, oz, bx, by, bz,
                                             H->err_flag, H->stream),
                 "coarse interpolation"));
+  if (covered) {
+    if (where == MG_MEM_HOST) CK(H, cudaStreamSynchronize(H->stream));
+    return MG_OK;
+  }
   int err = 0;
   CK(H, cudaMemcpyAsync(H->hscal, H->err_flag, sizeof(int), cudaMemcpyDeviceToHost, H->stream));
   CK(H, cudaStreamSynchronize(H->stream));

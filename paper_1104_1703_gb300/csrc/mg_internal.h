@@ -217,6 +217,8 @@ cudaError_t launch_u8_split_to_natural_bits(const Geom& g, uint8_t* const* code,
                                             cudaStream_t s);
 cudaError_t launch_fold_faces(const LevelDev& L0, const FineExtra& F, const double* bx, const double* by,
                               const double* bz, cudaStream_t s);
+// Boundary terms interpolated from the coarse potential, and L0.rhs =
+// h^2 rho - boundary terms.
 cudaError_t launch_fold_coarse(const LevelDev& L0, const FineExtra& F, const double* pc, int cnx, int cny,
                                int cnz, int ox, int oy, int oz, int* err_flag, cudaStream_t s);
 cudaError_t launch_combine_rhs(const LevelDev& L0, const FineExtra& F, cudaStream_t s);
