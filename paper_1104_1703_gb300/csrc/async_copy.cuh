@@ -124,6 +124,20 @@ __device__ __forceinline__ void tc_mma_f16(uint32_t d_tmem, uint64_t adesc, uint
       : "memory");
 }
 
+// The same with the descriptors as words: offsets within shared memory only
+// change the lower one.
+__device__ __forceinline__ void tc_mma_f16_words(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo,
+                                                 uint32_t b_hi, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\t"
+      "setp.ne.b32 p, %6, 0;\n\t"
+      "mov.b64 a, {%1, %2};\n\t"
+      "mov.b64 b, {%3, %4};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}" ::"r"(d_tmem),
+      "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
 // Arrives once on `bar` when every tcgen05 operation this thread issued
 // before it has completed (so their shared-memory operands may be reused and
 // their accumulators read).
@@ -155,6 +169,18 @@ __device__ __forceinline__ uint64_t smem_desc_kmajor(const void* base, uint32_t 
   const uint64_t a = smem_u32(base);
   return ((a >> 4) & 0x3fffull) | (((uint64_t)(lbo >> 4) & 0x3fffull) << 16) |
          (((uint64_t)(sbo >> 4) & 0x3fffull) << 32) | (1ull << 46);
+}
+
+// The same for a K-major operand in a swizzled layout, as a TMA copy with
+// that swizzle leaves it: rows of `span` bytes (32, 64 or 128) one after
+// another, 8 rows a group of `8 * span` bytes.  The pattern's address bits are
+// the absolute ones, so `base` may be any row of a buffer that is aligned to
+// the pattern (8 * span bytes) and any 32-byte step along K within the rows.
+__device__ __forceinline__ uint64_t smem_desc_swizzled(const void* base, uint32_t span) {
+  const uint64_t a = smem_u32(base);
+  const uint64_t type = span == 128 ? 2ull : (span == 64 ? 4ull : 6ull);
+  return ((a >> 4) & 0x3fffull) | (1ull << 16) | (((uint64_t)(8u * span >> 4) & 0x3fffull) << 32) | (1ull << 46) |
+         (type << 61);
 }
 
 // Shared-memory matrix descriptor of an operand in the canonical MN-major

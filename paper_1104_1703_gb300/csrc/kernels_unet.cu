@@ -1,20 +1,25 @@
 // Kernels of the learned initial guess's network: the 3x3x3 convolution as a
 // tcgen05 implicit GEMM, its weight gradients, and the packing of weights.
 //
-// Convolution.  An output tile is 128 voxels (a box of bx x by x bz) by cout
-// channels, accumulated in tensor memory (TMEM) in FP32 over K = 27 taps x
-// cin input channels.  Per 16 input channels one tcgen05.mma (kind::f16,
+// Convolution.  An output tile is 128 voxels by cout channels, accumulated in
+// tensor memory (TMEM) in FP32 over K = 27 taps x cin input channels; up to
+// four tiles (one box of voxels, one after another in it) are worked on
+// together: an MMA with few columns waits for the one before it on the same
+// accumulator (about 80 cycles at N = 16, of which 8 are work), so the tiles'
+// MMAs of one tap follow each other.  Per 16 input channels one tcgen05.mma (kind::f16,
 // BF16 x BF16 -> FP32, M = 128, N = cout) accumulates.  The A operand comes
 // from the channels-last input by TMA copies of a 5-D view of it,
-// (8 channels, x, y, z, channel chunk), landing in shared memory in the
-// canonical K-major layout (8-row x 16-byte core matrices); voxels outside
-// the grid read 0 (the convolution's zero padding).  Two ways to stage it:
-//  - halo rows (a tile that is one whole row of 128 voxels): one copy per 16
-//    input channels of the box (130 x 3 x 3) around the row; each of the 27
-//    taps is then a view of it, offset by (dz * 3 + dy) * 130 + dx rows, so
-//    the input is read once instead of 27 times;
+// (span channels, x, y, z, block of span channels), landing in shared memory
+// in the K-major layout swizzled over rows of span channels; voxels outside
+// the grid read 0 (the convolution's zero padding).  A row is as long as the
+// channels and the widest swizzle allow: 64, 32 or 16 channels.  Two ways to
+// stage it:
+//  - halo rows (tiles that are whole rows of 128 voxels): one copy per 16
+//    input channels of the box (130 x group + 2 x 3) around the group's rows;
+//    each of the 27 taps is then a view of it, so the input is read 4.5 times
+//    (group 4) instead of 27 times;
 //  - tap tiles (other shapes): one copy per tap and channel chunk of the
-//    tile's box shifted by the tap.
+//    group's box shifted by the tap.
 // The B operand (the weights, packed [27][cin / 8][cout][8]) stays resident
 // in shared memory for the whole launch when it fits (up to 72 KB), loaded
 // once per CTA by one bulk copy; otherwise it is staged with each tap.  The
@@ -65,18 +70,17 @@ __host__ __device__ ConvLayout conv_layout(const ConvArgs& a) {
   l.w_load = a.wres ? wall : 0u;
   l.w_bytes = a.wres ? (wall + 1023u) / 1024u * 1024u : 0u;
   if (a.halo) {
-    l.a_bytes = 2u * 9u * 130u * 16u;
+    l.a_bytes = 3u * (unsigned)(a.group + 2) * 130u * 32u;
     l.b_bytes = 0;
     l.units = a.cin / 16;
   } else {
-    l.a_bytes = (unsigned)a.kc * 2048u;
+    l.a_bytes = (unsigned)a.group * (unsigned)a.kc * 2048u;
     l.b_bytes = a.wres ? 0u : (unsigned)a.kc * (unsigned)a.cout * 16u;
     l.units = 27 * (a.cin / (8 * a.kc));
   }
-  // a TMA copy's shared-memory destination must be 128-byte aligned: the
-  // stages are laid out at a stride rounded up to 128 bytes (the weight
-  // stages' size, a multiple of 256, already is)
-  l.a_stride = (l.a_bytes + 127u) / 128u * 128u;
+  // a swizzled copy's shared-memory destination must be aligned to its
+  // pattern: the stages are laid out at a stride rounded up to 1024 bytes
+  l.a_stride = (l.a_bytes + 1023u) / 1024u * 1024u;
   return l;
 }
 
@@ -85,30 +89,69 @@ size_t conv_smem_bytes(const ConvArgs& a) {
   return 1024 + (size_t)l.w_bytes + (size_t)a.stages * (l.a_stride + l.b_bytes);
 }
 
-// Pipeline depth, resident weights and the halo path of a convolution: a
-// tile that is one full row of 128 voxels takes its input once with a halo
-// (box 130 x 3 x 3, every tap a view of it; this needs the weights
-// resident); weights up to 72 KB stay resident; as many stages as fit in
-// about 110 KB (two CTAs per multiprocessor) or, for halo stages, 220 KB.
-void conv_plan(ConvArgs& a) {
-  const unsigned wall = 27u * (unsigned)a.cin * (unsigned)a.cout * 2u;
-  a.wres = wall <= 72u * 1024u ? 1 : 0;
-  a.halo = (a.bx == 128 && a.wres) ? 1 : 0;
-  a.stages = 1;
-  const ConvLayout l = conv_layout(a);
-  const size_t per = l.a_stride + l.b_bytes;
-  const size_t budget = per > 12 * 1024 ? 220 * 1024 : 110 * 1024;
-  long long n = ((long long)budget - 1024 - (long long)l.w_bytes) / (long long)per;
-  if (n > kConvMaxStages) n = kConvMaxStages;
-  if (n < 2) n = 2;
-  a.stages = (int)n;
+// TMEM columns of a convolution CTA: two sets of `group` FP32 accumulators of
+// cout columns, rounded up to the power of two the allocator takes.
+__host__ __device__ uint32_t conv_tmem_cols(int group, int cout) {
+  const int c = 2 * group * cout;
+  return c <= 32 ? 32u : (c <= 64 ? 64u : (c <= 128 ? 128u : (c <= 256 ? 256u : 512u)));
 }
 
-// TMEM columns of a convolution CTA: two FP32 accumulators of cout columns,
-// rounded up to the power of two the allocator takes.
-__host__ __device__ uint32_t conv_tmem_cols(int cout) {
-  const int c = 2 * cout;
-  return c <= 32 ? 32u : (c <= 64 ? 64u : (c <= 128 ? 128u : (c <= 256 ? 256u : 512u)));
+namespace {
+
+// Channels per shared-memory row and 8-channel chunks per unit: the widest
+// row that divides the channels, and as many rows' blocks as make at most 64
+// channels.
+void conv_chunks(int cin, int* span, int* kc) {
+  *span = cin % 64 == 0 ? 64 : (cin % 32 == 0 ? 32 : 16);
+  const int blocks = cin / *span;
+  int n = 64 / *span;
+  while (blocks % n) --n;
+  *kc = n * *span / 8;
+}
+
+int conv_groups(const ConvArgs& a) {
+  return ((a.W + a.bx - 1) / a.bx) * ((a.H + a.by - 1) / a.by) * ((a.D + a.bz - 1) / a.bz);
+}
+
+}  // namespace
+
+// The plan of a convolution.  Weights up to 72 KB stay resident.  Tiles that
+// are whole rows of 128 voxels take the halo path (which needs resident
+// weights), four rows together where the level has them.  Otherwise as many
+// tiles are worked on together as leave about 100 groups, fit TMEM twice and
+// at least three stages in shared memory.
+void conv_plan(ConvArgs& a) {
+  constexpr size_t kBudget = 225 * 1024;  // dynamic shared memory
+  const unsigned wall = 27u * (unsigned)a.cin * (unsigned)a.cout * 2u;
+  a.wres = wall <= 72u * 1024u ? 1 : 0;
+  conv_chunks(a.cin, &a.span, &a.kc);
+  conv_tile_box(a.W, a.H, a.D, kConvTileM, &a.bx, &a.by, &a.bz);
+  a.halo = (a.bx == 128 && a.wres) ? 1 : 0;
+  auto stages = [&]() {
+    a.stages = 1;
+    const ConvLayout l = conv_layout(a);
+    const size_t per = l.a_stride + l.b_bytes, fixed = 1024 + (size_t)l.w_bytes;
+    const size_t n = fixed < kBudget ? (kBudget - fixed) / per : 0;
+    a.stages = n > (size_t)kConvMaxStages ? kConvMaxStages : (int)n;
+  };
+  for (a.group = 4; a.group >= 1; a.group /= 2) {
+    if (2 * a.group * a.cout > 512 && a.group > 1) continue;
+    if (a.halo) {
+      if (a.group > a.H && a.group > 1) continue;
+      a.span = 16;
+      a.kc = 2;
+      a.by = a.group;
+      a.bz = 1;
+    } else {
+      conv_tile_box(a.W, a.H, a.D, kConvTileM * a.group, &a.bx, &a.by, &a.bz);
+    }
+    stages();
+    if (a.group == 1 || (a.stages >= (a.halo ? 2 : 3) && (a.halo || conv_groups(a) >= 100))) break;
+  }
+  if (a.stages < 2) a.stages = 2;
+  a.ntx = (a.W + a.bx - 1) / a.bx;
+  a.nty = (a.H + a.by - 1) / a.by;
+  a.ntz = (a.D + a.bz - 1) / a.bz;
 }
 
 namespace {
@@ -127,7 +170,11 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   const int upt = a.cin / (8 * a.kc);
   const int NS = a.stages;
   const uint32_t acc_cols = (uint32_t)a.cout;
-  const uint32_t tcols = conv_tmem_cols(a.cout);
+  const uint32_t tcols = conv_tmem_cols(a.group, a.cout);
+  const int G = a.group;
+  __shared__ float bias_s[256];
+  if (a.bias)
+    for (int i = threadIdx.x; i < a.cout; i += kConvThreads) bias_s[i] = a.bias[i];
   if (threadIdx.x == 0) {
     for (int i = 0; i < NS; ++i) {
       mbar_init(&S.full[i], 1);
@@ -156,39 +203,58 @@ __global__ void __launch_bounds__(kConvThreads, 1)
         mbar_expect_tx(&S.wbar, lay.w_load);
         bulk_load(wres, a.w, lay.w_load, &S.wbar);
       }
-      int it = 0;
+      int it = 0, st = 0;
+      uint32_t ph = 1;  // parity of the wait for an empty stage: the first pass over the ring does not wait
       const bool stall = a.debug_stall && blockIdx.x == 0;
-      for (int t = blockIdx.x; t < ntiles && !*abort; t += gridDim.x) {
+      const int blocks = a.kc * 8 / a.span;
+      bool stop = false;
+      // waits for the next stage and arms it; false at an abort
+      auto acquire = [&]() {
+        if (it >= NS && !mbar_wait_bounded(&S.empty[st], ph, kConvLimitNs, abort)) {
+          atomicExch(a.err, 1);
+          *abort = 1;
+          return false;
+        }
+        if (stall && it >= NS) return false;  // stop issuing: the MMA thread's wait runs out
+        fence_proxy_async();
+        mbar_expect_tx(&S.full[st], lay.a_bytes + lay.b_bytes);
+        return true;
+      };
+      auto advance = [&]() {
+        ++it;
+        if (++st == NS) {
+          st = 0;
+          ph ^= 1u;
+        }
+      };
+      for (int t = blockIdx.x; t < ntiles && !stop && !*abort; t += gridDim.x) {
         const int tx = t % a.ntx, r = t / a.ntx, ty = r % a.nty, tz = r / a.nty;
         const int x0 = tx * a.bx, y0 = ty * a.by, z0 = tz * a.bz;
-        for (int u = 0; u < units; ++u, ++it) {
-          const int st = it % NS, n = it / NS;
-          if (n > 0 && !mbar_wait_bounded(&S.empty[st], (n - 1) & 1, kConvLimitNs, abort)) {
-            atomicExch(a.err, 1);
-            *abort = 1;
-            break;
+        if (a.halo) {
+          for (int u = 0; u < units && !stop; ++u) {
+            if ((stop = !acquire())) break;
+            // the group's rows of 128 output voxels with a one-voxel halo in
+            // x, y and z, 16 input channels: every tap is a view of it
+            tma_load_5d(stage_a + st * lay.a_stride, &map, 0, x0 - 1, y0 - 1, z0 - 1, u, &S.full[st]);
+            advance();
           }
-          if (stall && it >= NS) {  // stop issuing: the MMA thread's wait runs out
-            --it;
-            break;
-          }
-          fence_proxy_async();
-          mbar_expect_tx(&S.full[st], lay.a_bytes + lay.b_bytes);
-          if (a.halo) {
-            // the row of 128 output voxels with a one-voxel halo in x, y and
-            // z, 16 input channels: every tap is a view of it
-            tma_load_5d(stage_a + st * lay.a_stride, &map, 0, x0 - 1, y0 - 1, z0 - 1, 2 * u, &S.full[st]);
-          } else {
-            const int tap = u / upt, kq = u % upt;
-            const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-            tma_load_5d(stage_a + st * lay.a_stride, &map, 0, x0 + dx - 1, y0 + dy - 1, z0 + dz - 1, kq * a.kc,
-                        &S.full[st]);
-            if (lay.b_bytes)
-              bulk_load(stage_b + st * lay.b_bytes,
-                        a.w + ((size_t)tap * (a.cin / 8) + (size_t)kq * a.kc) * a.cout * 8, lay.b_bytes, &S.full[st]);
-          }
+        } else {
+          const __nv_bfloat16* w = a.w;
+#pragma unroll 1
+          for (int dz = -1; dz < 2 && !stop; ++dz)
+#pragma unroll 1
+            for (int dy = -1; dy < 2 && !stop; ++dy)
+#pragma unroll 1
+              for (int dx = -1; dx < 2 && !stop; ++dx)
+#pragma unroll 1
+                for (int q = 0; q < upt; ++q) {
+                  if ((stop = !acquire())) break;
+                  tma_load_5d(stage_a + st * lay.a_stride, &map, 0, x0 + dx, y0 + dy, z0 + dz, q * blocks, &S.full[st]);
+                  if (lay.b_bytes) bulk_load(stage_b + st * lay.b_bytes, w, lay.b_bytes, &S.full[st]);
+                  w += (size_t)a.kc * a.cout * 8;
+                  advance();
+                }
         }
-        if (stall) break;
       }
       // at an abort, let the copies still in flight land before the CTA exits
       if (*abort) {
@@ -200,9 +266,25 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   } else if (warp == 1) {
     if (lane == 0) {
       // ---- MMAs ----
+      // One thread issues them all, so whatever it computes per MMA bounds
+      // the kernel (divisions per tap and whole descriptors: 2800 cycles per
+      // tile of a 16 -> 16 layer): the taps of a group of four are unrolled
+      // and descriptors advance by additions to their lower word.
       const uint32_t idesc = idesc_bf16_f32(kConvTileM, a.cout);
       const uint32_t wchunk = (uint32_t)a.cout * 16u;  // bytes of one 8-channel chunk of one tap's weights
-      int it = 0, tc = 0;
+      const uint32_t wtap = (uint32_t)(a.cin / 8) * wchunk >> 4;  // one tap's weights, in descriptor units of 16 bytes
+      const int ksteps = a.kc / 2;
+      // a tile's 128 rows of a block are 256 * span bytes, the tiles' of one
+      // block follow each other; 16 channels on are 32 bytes within the rows,
+      // or the next block
+      const uint32_t tstep = 16u * (uint32_t)a.span;
+      const uint32_t bstep = a.span == 16 ? (uint32_t)G * 256u : 2u;
+      const uint64_t adesc = smem_desc_swizzled(stage_a, 2 * a.span);
+      const uint64_t wdesc = smem_desc_kmajor(lay.w_bytes ? wres : stage_b, wchunk, 128);
+      const uint32_t ahi = (uint32_t)(adesc >> 32), bhi = (uint32_t)(wdesc >> 32);
+      const uint32_t arow = (uint32_t)(G + 2) * 260u;  // halo path: one plane of the box
+      int it = 0, st = 0, tc = 0;
+      uint32_t ph = 0;
       bool issued = false;
       if (lay.w_bytes && !mbar_wait_bounded(&S.wbar, 0, kConvLimitNs, abort)) {
         atomicExch(a.err, 1);
@@ -216,11 +298,11 @@ __global__ void __launch_bounds__(kConvThreads, 1)
           break;
         }
         tc_fence_after();
-        const uint32_t d = tmem + (uint32_t)b * acc_cols;
+        const uint32_t d = tmem + (uint32_t)(b * G) * acc_cols;
+        uint32_t wlo = (uint32_t)wdesc;  // resident weights: the unit's, in copy order
         bool ok = true;
-        for (int u = 0; u < units; ++u, ++it) {
-          const int st = it % NS;
-          if (!mbar_wait_bounded(&S.full[st], (it / NS) & 1, kConvLimitNs, abort)) {
+        for (int u = 0; u < units; ++u) {
+          if (!mbar_wait_bounded(&S.full[st], ph, kConvLimitNs, abort)) {
             atomicExch(a.err, 1);
             *abort = 1;
             ok = false;
@@ -228,29 +310,64 @@ __global__ void __launch_bounds__(kConvThreads, 1)
           }
           S.consumed = it + 1;
           tc_fence_after();
-          const unsigned char* A = stage_a + st * lay.a_stride;
+          const uint32_t alo = (uint32_t)adesc + (uint32_t)st * (lay.a_stride >> 4);
           if (a.halo) {
-            // channels 16u .. 16u + 15 of the 27 taps: each tap's 128 rows
-            // start (dz, dy, dx) rows into the halo box; the box's rows are
-            // 16 bytes apart and its two 8-channel chunks 9 x 130 rows apart
-            for (int tap = 0; tap < 27; ++tap) {
-              const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-              const uint64_t ad = smem_desc_kmajor(A + ((dz * 3 + dy) * 130 + dx) * 16, 9u * 130u * 16u, 128);
-              const uint64_t bd = smem_desc_kmajor(wres + ((size_t)tap * (a.cin / 8) + 2 * u) * wchunk, wchunk, 128);
-              tc_mma_f16(d, ad, bd, idesc, (u > 0 || tap > 0) ? 1u : 0u);
+            // channels 16u .. 16u + 15 of the 27 taps: a tile's 128 rows
+            // start (dz, tile + dy, dx) rows of 32 bytes into the halo box
+            uint32_t blo = wlo + (uint32_t)(2 * u) * (wchunk >> 4);
+            uint32_t acc = u > 0 ? 1u : 0u;
+            uint32_t plane = alo;
+#pragma unroll 1
+            for (int dz = 0; dz < 3; ++dz, plane += arow) {
+              if (G == 4) {
+#pragma unroll
+                for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+                  for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll
+                    for (int g = 0; g < 4; ++g)
+                      tc_mma_f16_words(d + (uint32_t)g * acc_cols, plane + (uint32_t)((g + dy) * 260 + dx * 2), ahi, blo,
+                                       bhi, idesc, acc);
+                    acc = 1u;
+                    blo += wtap;
+                  }
+              } else {
+#pragma unroll 1
+                for (int dy = 0; dy < 3; ++dy)
+#pragma unroll 1
+                  for (int dx = 0; dx < 3; ++dx) {
+#pragma unroll 1
+                    for (int g = 0; g < G; ++g)
+                      tc_mma_f16_words(d + (uint32_t)g * acc_cols, plane + (uint32_t)((g + dy) * 260 + dx * 2), ahi, blo,
+                                       bhi, idesc, acc);
+                    acc = 1u;
+                    blo += wtap;
+                  }
+              }
             }
           } else {
-            const int tap = u / upt, kq = u % upt;
-            const unsigned char* Bm = lay.w_bytes ? wres + ((size_t)tap * (a.cin / 8) + (size_t)kq * a.kc) * wchunk
-                                                  : stage_b + st * lay.b_bytes;
-            for (int ks = 0; ks < a.kc / 2; ++ks) {
-              const uint64_t ad = smem_desc_kmajor(A + ks * 2 * 2048, 2048, 128);
-              const uint64_t bd = smem_desc_kmajor(Bm + ks * 2 * wchunk, wchunk, 128);
-              tc_mma_f16(d, ad, bd, idesc, (u > 0 || ks > 0) ? 1u : 0u);
+            uint32_t blo = lay.w_bytes ? wlo : (uint32_t)wdesc + (uint32_t)st * (lay.b_bytes >> 4);
+#pragma unroll 1
+            for (int ks = 0; ks < ksteps; ++ks) {
+              const uint32_t al = alo + (uint32_t)ks * bstep;
+              const uint32_t acc = (u > 0 || ks > 0) ? 1u : 0u;
+              tc_mma_f16_words(d, al, ahi, blo, bhi, idesc, acc);
+              if (G > 1) tc_mma_f16_words(d + acc_cols, al + tstep, ahi, blo, bhi, idesc, acc);
+              if (G > 2) {
+                tc_mma_f16_words(d + 2 * acc_cols, al + 2 * tstep, ahi, blo, bhi, idesc, acc);
+                tc_mma_f16_words(d + 3 * acc_cols, al + 3 * tstep, ahi, blo, bhi, idesc, acc);
+              }
+              blo += 2u * wchunk >> 4;
             }
+            wlo += (uint32_t)a.kc * (wchunk >> 4);
           }
           tc_commit(&S.empty[st]);
           issued = true;
+          ++it;
+          if (++st == NS) {
+            st = 0;
+            ph ^= 1u;
+          }
         }
         if (!ok) break;
         tc_commit(&S.accf[b]);
@@ -264,8 +381,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   } else {
     // ---- epilogue: warps 2..5 own TMEM lane quarters 2, 3, 0, 1 ----
     const int q = warp & 3;
-    const int m = 32 * q + lane;
-    const int mx = m % a.bx, my = (m / a.bx) % a.by, mz = m / (a.bx * a.by);
+    const int lbx = __ffs(a.bx) - 1, lby = __ffs(a.by) - 1;
     int tc = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++tc) {
       const int b = tc & 1, n = tc >> 1;
@@ -284,25 +400,33 @@ __global__ void __launch_bounds__(kConvThreads, 1)
       __syncwarp();
       tc_fence_after();
       const int tx = t % a.ntx, r = t / a.ntx, ty = r % a.nty, tz = r / a.nty;
-      const int x = tx * a.bx + mx, y = ty * a.by + my, z = tz * a.bz + mz;
-      const bool in = x < a.W && y < a.H && z < a.D;
-      const size_t v = ((size_t)z * a.H + y) * a.W + x;
-      for (int c0 = 0; c0 < a.cout; c0 += 16) {
+      for (int gc = 0; gc < G * a.cout; gc += 16) {
+        const int g = gc / a.cout, c0 = gc - g * a.cout;
+        const int m = g * kConvTileM + 32 * q + lane;  // the boxes' sides are powers of two
+        const int mx = m & (a.bx - 1), mr = m >> lbx;
+        const int x = tx * a.bx + mx, y = ty * a.by + (mr & (a.by - 1)), z = tz * a.bz + (mr >> lby);
+        const bool in = x < a.W && y < a.H && z < a.D;
+        const size_t v = ((size_t)z * a.H + y) * a.W + x;
         float val[16];
-        tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)b * acc_cols + (uint32_t)c0, val);
+        tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * G) * acc_cols + (uint32_t)gc, val);
         if (!in) continue;
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
           float f = val[i];
-          if (a.bias) f += a.bias[c0 + i];
+          if (a.bias) f += bias_s[c0 + i];
           if (a.relu) f = fmaxf(f, 0.0f);
           val[i] = f;
         }
-        if (a.mask) {
-          const __nv_bfloat16* mk = a.mask + v * a.mask_stride + a.mask_off + c0;
+        if (a.mask) {  // 16 channels of a voxel: 32 aligned bytes
+          const uint4* mk = reinterpret_cast<const uint4*>(a.mask + v * a.mask_stride + a.mask_off + c0);
+          const uint4 m0 = mk[0], m1 = mk[1];
+          const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
 #pragma unroll
-          for (int i = 0; i < 16; ++i)
-            if (!(__bfloat162float(mk[i]) > 0.0f)) val[i] = 0.0f;
+          for (int i = 0; i < 16; ++i) {
+            // BF16 > 0: the value's bits as an FP32's upper half
+            const uint32_t hb = (i & 1) ? mw[i >> 1] & 0xffff0000u : mw[i >> 1] << 16;
+            if (!(__uint_as_float(hb) > 0.0f)) val[i] = 0.0f;
+          }
         }
         if (a.out_f32) {
           float* o = a.out_f32 + v * a.cout + c0;
@@ -355,32 +479,22 @@ __global__ void pack_weights_kernel(const float* __restrict__ w, int cout, int c
 
 }  // namespace
 
-int conv_kc(int cin) {
-  const int chunks = cin / 8;
-  for (int k = 8; k >= 2; k -= 2)
-    if (chunks % k == 0) return k;
-  return 2;
-}
-
-
-
-
 cudaError_t init_conv_kernel(size_t smem_bytes) {
   return cudaFuncSetAttribute(conv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
 }
 
-// The output tile's box: powers of two with bx * by * bz = 128 exactly (the
-// copy of a tile must deliver the 128 rows the MMA and the barrier's byte
-// count expect; rows beyond the grid read 0 and are not stored).
-void conv_tile_box(int W, int H, int D, int* bx, int* by, int* bz) {
+// Powers of two with bx * by * bz = voxels exactly (the copy of a box must
+// deliver the rows the MMAs and the barrier's byte count expect; rows beyond
+// the grid read 0 and are not stored).
+void conv_tile_box(int W, int H, int D, int voxels, int* bx, int* by, int* bz) {
   auto pow2_at_most = [](int n, int cap) {
     int p = 1;
     while (2 * p <= n && 2 * p <= cap) p *= 2;
     return p;
   };
   *bx = pow2_at_most(W, 128);
-  *by = pow2_at_most(H, 128 / *bx);
-  *bz = 128 / (*bx * *by);
+  *by = pow2_at_most(H, voxels / *bx);
+  *bz = voxels / (*bx * *by);
   (void)D;
 }
 
@@ -398,17 +512,27 @@ PFN_cuTensorMapEncodeTiled_v12000 conv_encode_fn() {
 }
 }  // namespace
 
-bool make_conv_input_map(CUtensorMap* map, const __nv_bfloat16* x, int W, int H, int D, int cin, int bx, int by,
-                         int bz, int kc) {
+bool make_conv_input_map(CUtensorMap* map, const __nv_bfloat16* x, int W, int H, int D, int cin, int span, int bx,
+                         int by, int bz, int blocks) {
   PFN_cuTensorMapEncodeTiled_v12000 fn = conv_encode_fn();
   if (!fn) return false;
-  const cuuint64_t dims[5] = {8, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)D, (cuuint64_t)(cin / 8)};
-  const cuuint64_t strides[4] = {(cuuint64_t)cin * 2, (cuuint64_t)W * cin * 2, (cuuint64_t)H * W * cin * 2, 16};
-  const cuuint32_t box[5] = {8, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz, (cuuint32_t)kc};
+  const cuuint64_t dims[5] = {(cuuint64_t)span, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)D, (cuuint64_t)(cin / span)};
+  const cuuint64_t strides[4] = {(cuuint64_t)cin * 2, (cuuint64_t)W * cin * 2, (cuuint64_t)H * W * cin * 2,
+                                 (cuuint64_t)span * 2};
+  const cuuint32_t box[5] = {(cuuint32_t)span, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz, (cuuint32_t)blocks};
+  const CUtensorMapSwizzle sw = span == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+                                : span == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                : span == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
+                                             : CU_TENSOR_MAP_SWIZZLE_NONE;
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)x, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+            sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
          CUDA_SUCCESS;
+}
+
+bool make_conv_map(CUtensorMap* map, const __nv_bfloat16* x, const ConvArgs& a) {
+  if (a.halo) return make_conv_input_map(map, x, a.W, a.H, a.D, a.cin, 16, 130, a.group + 2, 3, 1);
+  return make_conv_input_map(map, x, a.W, a.H, a.D, a.cin, a.span, a.bx, a.by, a.bz, a.kc * 8 / a.span);
 }
 
 int conv_grid(const ConvArgs& a, size_t smem_bytes) {
@@ -418,7 +542,7 @@ int conv_grid(const ConvArgs& a, size_t smem_bytes) {
     (void)cudaGetLastError();
     per_sm = 1;
   }
-  const int by_tmem = (int)(512 / conv_tmem_cols(a.cout));
+  const int by_tmem = (int)(512 / conv_tmem_cols(a.group, a.cout));
   if (per_sm > by_tmem) per_sm = by_tmem;
   const int tiles = a.ntx * a.nty * a.ntz;
   const int g = per_sm * device_sms();

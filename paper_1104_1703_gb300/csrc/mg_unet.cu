@@ -168,9 +168,6 @@ std::string conv_name(const mg_unet* N, int i) {
 }
 
 mg_status setup_conv(mg_unet* N, Conv& C) {
-  int bx, by, bz;
-  conv_tile_box(C.in.W, C.in.H, C.in.D, &bx, &by, &bz);
-  const int kc = conv_kc(C.cin_pad);
   ConvArgs& a = C.args;
   std::memset(&a, 0, sizeof(a));
   a.W = C.in.W;
@@ -178,13 +175,6 @@ mg_status setup_conv(mg_unet* N, Conv& C) {
   a.D = C.in.D;
   a.cin = C.cin_pad;
   a.cout = C.cout;
-  a.kc = kc;
-  a.bx = bx;
-  a.by = by;
-  a.bz = bz;
-  a.ntx = (a.W + bx - 1) / bx;
-  a.nty = (a.H + by - 1) / by;
-  a.ntz = (a.D + bz - 1) / bz;
   a.w = C.wf;
   a.bias = C.b;
   a.relu = 1;
@@ -194,8 +184,7 @@ mg_status setup_conv(mg_unet* N, Conv& C) {
   a.err = N->err;
   conv_plan(a);
   C.smem = conv_smem_bytes(a);
-  if (!(a.halo ? make_conv_input_map(&C.map_in, C.in.p, a.W, a.H, a.D, a.cin, 130, 3, 3, 2)
-               : make_conv_input_map(&C.map_in, C.in.p, a.W, a.H, a.D, a.cin, bx, by, bz, kc)))
+  if (!make_conv_map(&C.map_in, C.in.p, a))
     return ufail(N, MG_ERR_CUDA, "tensor map of a convolution input was refused");
   return MG_OK;
 }
@@ -205,11 +194,11 @@ mg_status setup_conv(mg_unet* N, Conv& C) {
 // a ReLU output) and the weight gradient's tensor maps and partition.
 mg_status setup_conv_backward(mg_unet* N, Conv& C, const Tensor* to, const Tensor* mask) {
   int bx, by, bz;
-  conv_tile_box(C.in.W, C.in.H, C.in.D, &bx, &by, &bz);
+  conv_tile_box(C.in.W, C.in.H, C.in.D, kConvTileM, &bx, &by, &bz);
   const int T = ((C.in.W + bx - 1) / bx) * ((C.in.H + by - 1) / by) * ((C.in.D + bz - 1) / bz);
   // weight gradient
-  if (!make_conv_input_map(&C.map_x1, C.in.p, C.in.W, C.in.H, C.in.D, C.cin_pad, bx, by, bz, 1) ||
-      !make_conv_input_map(&C.map_g, C.gz.p, C.gz.W, C.gz.H, C.gz.D, C.cout, bx, by, bz, C.cout / 8))
+  if (!make_conv_input_map(&C.map_x1, C.in.p, C.in.W, C.in.H, C.in.D, C.cin_pad, 8, bx, by, bz, 1) ||
+      !make_conv_input_map(&C.map_g, C.gz.p, C.gz.W, C.gz.H, C.gz.D, C.cout, 8, bx, by, bz, C.cout / 8))
     return ufail(N, MG_ERR_CUDA, "tensor map of a weight gradient was refused");
   WgradArgs& w = C.wg;
   std::memset(&w, 0, sizeof(w));
@@ -232,7 +221,6 @@ mg_status setup_conv_backward(mg_unet* N, Conv& C, const Tensor* to, const Tenso
   w.err = N->err;
   if (!to) return MG_OK;
   // backward data: K = cout (the gradient's channels), N = cin_pad
-  const int kc = conv_kc(C.cout);
   ConvArgs& a = C.bargs;
   std::memset(&a, 0, sizeof(a));
   a.W = C.in.W;
@@ -240,13 +228,6 @@ mg_status setup_conv_backward(mg_unet* N, Conv& C, const Tensor* to, const Tenso
   a.D = C.in.D;
   a.cin = C.cout;
   a.cout = C.cin_pad;
-  a.kc = kc;
-  a.bx = bx;
-  a.by = by;
-  a.bz = bz;
-  a.ntx = w.ntx;
-  a.nty = w.nty;
-  a.ntz = w.ntz;
   a.w = C.wb;
   a.bias = nullptr;
   a.relu = 0;
@@ -261,8 +242,7 @@ mg_status setup_conv_backward(mg_unet* N, Conv& C, const Tensor* to, const Tenso
   a.err = N->err;
   conv_plan(a);
   C.bsmem = conv_smem_bytes(a);
-  if (!(a.halo ? make_conv_input_map(&C.map_gz_bd, C.gz.p, a.W, a.H, a.D, a.cin, 130, 3, 3, 2)
-               : make_conv_input_map(&C.map_gz_bd, C.gz.p, a.W, a.H, a.D, a.cin, bx, by, bz, kc)))
+  if (!make_conv_map(&C.map_gz_bd, C.gz.p, a))
     return ufail(N, MG_ERR_CUDA, "tensor map of a backward convolution was refused");
   return MG_OK;
 }
@@ -512,7 +492,7 @@ mg_status mg_unet_create(int levels, int base, int nx, int ny, int nz, void* cud
     o_gz[i] = R.take(sizeof(__nv_bfloat16) * (size_t)Vl * C.cout);
     // weight-gradient partial sums (the partition of setup_conv_backward)
     int bx, by, bz;
-    conv_tile_box(nx >> l, ny >> l, nz >> l, &bx, &by, &bz);
+    conv_tile_box(nx >> l, ny >> l, nz >> l, kConvTileM, &bx, &by, &bz);
     const int T = (((nx >> l) + bx - 1) / bx) * (((ny >> l) + by - 1) / by) * (((nz >> l) + bz - 1) / bz);
     const int nmblk = (27 * C.cin_pad + 127) / 128;
     int ns = (2 * device_sms()) / nmblk;

@@ -19,15 +19,18 @@ constexpr int kConvThreads = 192;  // warp 0 copies, warp 1 issues the MMAs, war
 constexpr int kConvMaxStages = 16;
 constexpr int kConvTileM = 128;    // voxels per output tile (the MMA's M)
 
-// One 3x3x3 convolution (zero padding 1) as an implicit GEMM: output tile of
-// 128 voxels x cout channels, K = 27 taps x cin channels.  The pipeline's
-// unit is one tap and `kc` 8-channel chunks of the input.
+// One 3x3x3 convolution (zero padding 1) as an implicit GEMM: output tiles of
+// 128 voxels x cout channels, K = 27 taps x cin channels, `group` tiles at a
+// time.  The pipeline's unit is one tap and `kc` 8-channel chunks of the
+// group's input.
 struct ConvArgs {
   int W, H, D;           // spatial size of input and output
   int cin, cout;         // channels, multiples of 16; cout <= 256
-  int kc;                // 8-channel chunks per unit (even, divides cin / 8, <= 8)
-  int bx, by, bz;        // the output tile's box (bx * by * bz = 128)
-  int ntx, nty, ntz;     // tiles per axis
+  int kc;                // 8-channel chunks per unit (a multiple of span / 8, divides cin / 8, <= 8)
+  int span;              // channels per shared-memory row: 64, 32 or 16 (128-, 64- or 32-byte swizzle)
+  int group;             // tiles worked on together, 1, 2 or 4
+  int bx, by, bz;        // the group's box (bx * by * bz = 128 * group, tiles one after another)
+  int ntx, nty, ntz;     // groups per axis
   const __nv_bfloat16* w;  // packed weights [27][cin / 8][cout][8]
   const float* bias;       // nullable, [cout]
   int relu;                // apply max(0, .) after the bias
@@ -50,22 +53,25 @@ struct ConvLayout {
   unsigned w_load;   // bytes of the packed weights copied in once (a multiple of 16)
   unsigned w_bytes;  // their shared-memory footprint, rounded to 1 KB (0: staged per unit)
   unsigned a_bytes;  // input bytes per unit (the copy's size)
-  unsigned a_stride; // their shared-memory stride, a multiple of 128 bytes
+  unsigned a_stride; // their shared-memory stride, a multiple of 1024 bytes (the widest swizzle pattern)
   unsigned b_bytes;  // weight bytes per unit
   int units;         // units per tile
 };
 __host__ __device__ ConvLayout conv_layout(const ConvArgs& a);
+// Everything but the pointers from a's W, H, D, cin and cout.
 void conv_plan(ConvArgs& a);
 size_t conv_smem_bytes(const ConvArgs& a);
 
-__host__ __device__ uint32_t conv_tmem_cols(int cout);
-int conv_kc(int cin);
+__host__ __device__ uint32_t conv_tmem_cols(int group, int cout);
 cudaError_t init_conv_kernel(size_t smem_bytes);
-// `map` describes the input tensor: dims (8, W, H, D, cin / 8), box
-// (8, bx, by, bz, kc), BF16; for the halo path box (8, 130, 3, 3, 2).
-bool make_conv_input_map(CUtensorMap* map, const __nv_bfloat16* x, int W, int H, int D, int cin, int bx, int by,
-                         int bz, int kc);
-void conv_tile_box(int W, int H, int D, int* bx, int* by, int* bz);
+// `map` describes the input tensor: dims (span, W, H, D, cin / span), box
+// (span, bx, by, bz, blocks), BF16, swizzled over rows of `span` channels
+// (span 8: no swizzle).
+bool make_conv_input_map(CUtensorMap* map, const __nv_bfloat16* x, int W, int H, int D, int cin, int span, int bx,
+                         int by, int bz, int blocks);
+bool make_conv_map(CUtensorMap* map, const __nv_bfloat16* x, const ConvArgs& a);
+// Box of `voxels` (a power of two) voxels, powers of two per axis.
+void conv_tile_box(int W, int H, int D, int voxels, int* bx, int* by, int* bz);
 cudaError_t launch_conv(const CUtensorMap& map, const ConvArgs& a, int grid, cudaStream_t s);
 int conv_grid(const ConvArgs& a, size_t smem_bytes);
 
