@@ -183,12 +183,15 @@ __device__ __forceinline__ uint64_t smem_desc_swizzled(const void* base, uint32_
          (type << 61);
 }
 
-// Shared-memory matrix descriptor of an operand in the canonical MN-major
-// layout without swizzle: core matrices of 8 K-rows x 16 bytes (8 M or N
-// elements) stored as 128 contiguous bytes; `lbo` is the byte distance
-// between core matrices adjacent along K, `sbo` along M (or N).
-__device__ __forceinline__ uint64_t smem_desc_mnmajor(const void* base, uint32_t lbo, uint32_t sbo) {
-  return smem_desc_kmajor(base, lbo, sbo);
+// Shared-memory matrix descriptor of an MN-major operand in a swizzled layout:
+// rows (K) of `span` bytes of M or N elements, 8 rows a group, groups one after another along K; `next` is the byte
+// distance between blocks of span bytes adjacent along M (or N).  (Here the
+// first offset field is the M or N distance and the second the K distance.)
+__device__ __forceinline__ uint64_t smem_desc_mn_swizzled(const void* base, uint32_t span, uint32_t next) {
+  const uint64_t a = smem_u32(base);
+  const uint64_t type = span == 128 ? 2ull : (span == 64 ? 4ull : 6ull);
+  return ((a >> 4) & 0x3fffull) | (((uint64_t)(next >> 4) & 0x3fffull) << 16) |
+         (((uint64_t)(8u * span >> 4) & 0x3fffull) << 32) | (1ull << 46) | (type << 61);
 }
 
 // Instruction descriptor of kind::f16 with BF16 A and B, FP32 accumulator,

@@ -587,45 +587,83 @@ __global__ void input_to_bf16_kernel(const float* __restrict__ x, long long V, _
   }
 }
 
+// The kernels below take 8 channels (16 bytes) of a voxel per thread; those on
+// two grid levels take a row (y, z) per block round, so a thread's place costs
+// one 32-bit division (with a 64-bit division per channel they took 2 to 7
+// times the time of their bytes).
+__device__ __forceinline__ void unpack8(const uint4& r, float* f) {
+  const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    f[2 * i] = __uint_as_float(w[i] << 16);
+    f[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+  }
+}
+
+__device__ __forceinline__ uint4 pack8(const float* f) {
+  __align__(16) __nv_bfloat16 o[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) o[i] = __float2bfloat16_rn(f[i]);
+  return *reinterpret_cast<const uint4*>(o);
+}
+
+__device__ __forceinline__ uint4 load8(const __nv_bfloat16* p) { return *reinterpret_cast<const uint4*>(p); }
+
+// Sum over the 8 children (2x, 2y, 2z) .. of 8 channels at channel offset
+// `ch` of a tensor of twice the size, in the order z, y, x.
+__device__ __forceinline__ void child_sum8(const __nv_bfloat16* __restrict__ src, int stride, int ch, int W, int H, int x,
+                                           int y, int z, float* acc) {
+  uint4 r[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const long long vs = ((long long)(2 * z + (k >> 2)) * (2 * H) + (2 * y + ((k >> 1) & 1))) * (2 * W) + (2 * x + (k & 1));
+    r[k] = load8(src + vs * stride + ch);
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) acc[i] = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    float f[8];
+    unpack8(r[k], f);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] += f[i];
+  }
+}
+
 // 2x2x2 mean of src (level size 2W x 2H x 2D, channel stride ss, offset so)
-// into dst (W x H x D, c channels, stride ds, offset do); one thread per
-// output voxel and group of 8 channels
+// into dst (W x H x D, c channels, stride ds, offset do)
 __global__ void avg_pool_kernel(const __nv_bfloat16* __restrict__ src, int ss, int so, int W, int H, int D, int c,
                                 __nv_bfloat16* __restrict__ dst, int ds, int dofs) {
-  const long long n = (long long)W * H * D * (c / 8);
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const int g = (int)(e % (c / 8));
-    const long long v = e / (c / 8);
-    const int x = (int)(v % W), y = (int)((v / W) % H), z = (int)(v / ((long long)W * H));
-    float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int dz = 0; dz < 2; ++dz)
-      for (int dy = 0; dy < 2; ++dy)
-        for (int dx = 0; dx < 2; ++dx) {
-          const long long vs = ((long long)(2 * z + dz) * (2 * H) + (2 * y + dy)) * (2 * W) + (2 * x + dx);
-          const uint4 raw = *reinterpret_cast<const uint4*>(src + vs * ss + so + 8 * g);
-          const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&raw);
+  const int G = c / 8;
+  for (int row = blockIdx.x; row < H * D; row += gridDim.x) {
+    const int z = row / H, y = row - z * H;
+    for (int e = threadIdx.x; e < W * G; e += blockDim.x) {
+      const int x = e / G, g = e - x * G;
+      float acc[8];
+      child_sum8(src, ss, so + 8 * g, W, H, x, y, z, acc);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) acc[i] += __bfloat162float(h[i]);
-        }
-    __align__(16) __nv_bfloat16 o[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) o[i] = __float2bfloat16_rn(acc[i] * 0.125f);
-    *reinterpret_cast<uint4*>(dst + v * ds + dofs + 8 * g) = *reinterpret_cast<const uint4*>(o);
+      for (int i = 0; i < 8; ++i) acc[i] *= 0.125f;
+      *reinterpret_cast<uint4*>(dst + ((long long)row * W + x) * ds + dofs + 8 * g) = pack8(acc);
+    }
   }
 }
 
 // nearest-neighbour upsampling by 2 of src (W x H x D, c channels, stride ss,
-// offset so) into dst (2W x 2H x 2D, stride ds, offset do)
+// offset so) into dst (2W x 2H x 2D, stride ds, offset do); a block round per
+// output row
 __global__ void upsample_kernel(const __nv_bfloat16* __restrict__ src, int ss, int so, int W, int H, int D, int c,
                                 __nv_bfloat16* __restrict__ dst, int ds, int dofs) {
-  const long long n = 8LL * W * H * D * (c / 8);
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const int g = (int)(e % (c / 8));
-    const long long v = e / (c / 8);
-    const int X = 2 * W, Y = 2 * H;
-    const int x = (int)(v % X), y = (int)((v / X) % Y), z = (int)(v / ((long long)X * Y));
-    const long long vs = ((long long)(z >> 1) * H + (y >> 1)) * W + (x >> 1);
-    *reinterpret_cast<uint4*>(dst + v * ds + dofs + 8 * g) = *reinterpret_cast<const uint4*>(src + vs * ss + so + 8 * g);
+  const int G = c / 8;
+  for (int row = blockIdx.x; row < 4 * H * D; row += gridDim.x) {
+    const int z = row / (2 * H), y = row - z * (2 * H);
+    const __nv_bfloat16* s = src + ((long long)(z >> 1) * H + (y >> 1)) * W * ss + so;
+    __nv_bfloat16* o = dst + (long long)row * (2 * W) * ds + dofs;
+    for (int e = threadIdx.x; e < W * G; e += blockDim.x) {
+      const int x = e / G, g = e - x * G;
+      const uint4 v = load8(s + (long long)x * ss + 8 * g);
+      *reinterpret_cast<uint4*>(o + (long long)(2 * x) * ds + 8 * g) = v;
+      *reinterpret_cast<uint4*>(o + (long long)(2 * x + 1) * ds + 8 * g) = v;
+    }
   }
 }
 
@@ -634,10 +672,19 @@ __global__ void upsample_kernel(const __nv_bfloat16* __restrict__ src, int ss, i
 __global__ void head_kernel(const __nv_bfloat16* __restrict__ u, int c, const float* __restrict__ w,
                             const float* __restrict__ b, const __nv_bfloat16* __restrict__ x0, long long V,
                             float* __restrict__ pred) {
+  __shared__ float ws[128];
+  for (int i = threadIdx.x; i < c; i += blockDim.x) ws[i] = w[i];
+  __syncthreads();
   for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
+    const uint32_t m = *reinterpret_cast<const uint32_t*>(x0 + v * 16);  // channels 0 and 1
     float acc = b[0];
-    for (int i = 0; i < c; ++i) acc = fmaf(w[i], __bfloat162float(u[v * c + i]), acc);
-    pred[v] = __bfloat162float(x0[v * 16 + 1]) > 0.0f ? acc : 0.0f;
+    for (int i = 0; i < c; i += 8) {
+      float f[8];
+      unpack8(load8(u + v * c + i), f);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) acc = fmaf(ws[i + k], f[k], acc);
+    }
+    pred[v] = __uint_as_float(m & 0xffff0000u) > 0.0f ? acc : 0.0f;
   }
 }
 
@@ -659,6 +706,12 @@ int ew_grid(long long n) {
   return b < 1 ? 1 : (int)b;
 }
 
+// blocks of a kernel that takes a row per block round
+int row_grid(long long rows) {
+  const long long cap = 16LL * device_sms();
+  return rows > cap ? (int)cap : (rows < 1 ? 1 : (int)rows);
+}
+
 }  // namespace
 
 cudaError_t launch_input_to_bf16(const float* x, long long V, __nv_bfloat16* out, cudaStream_t s) {
@@ -670,14 +723,14 @@ cudaError_t launch_input_to_bf16(const float* x, long long V, __nv_bfloat16* out
 cudaError_t launch_avg_pool(const __nv_bfloat16* src, int ss, int so, int W, int H, int D, int c, __nv_bfloat16* dst,
                             int ds, int dofs, cudaStream_t s) {
   count_launch();
-  avg_pool_kernel<<<ew_grid((long long)W * H * D * (c / 8)), 256, 0, s>>>(src, ss, so, W, H, D, c, dst, ds, dofs);
+  avg_pool_kernel<<<row_grid((long long)H * D), 256, 0, s>>>(src, ss, so, W, H, D, c, dst, ds, dofs);
   return cudaGetLastError();
 }
 
 cudaError_t launch_upsample(const __nv_bfloat16* src, int ss, int so, int W, int H, int D, int c, __nv_bfloat16* dst,
                             int ds, int dofs, cudaStream_t s) {
   count_launch();
-  upsample_kernel<<<ew_grid(8LL * W * H * D * (c / 8)), 256, 0, s>>>(src, ss, so, W, H, D, c, dst, ds, dofs);
+  upsample_kernel<<<row_grid(4LL * H * D), 256, 0, s>>>(src, ss, so, W, H, D, c, dst, ds, dofs);
   return cudaGetLastError();
 }
 
@@ -705,22 +758,36 @@ cudaError_t launch_tensor_to_natural(const __nv_bfloat16* t, int stride, int off
 // Weight gradient of a convolution: dW[o][i][tap] = sum over voxels v of
 // g[v][o] x[v + offset(tap)][i], with g the gradient of the pre-activation
 // and x the layer's input (zero outside the grid).  As a GEMM: rows (tap, i)
-// of the tap-major row space (27 x cin rows), columns o, K = the voxels.  A
-// CTA takes 128 rows and a range of voxel tiles: per tile, the 16 channel
-// octets of its rows are 16 TMA copies of the input tile shifted by each
-// octet's tap (box 8 channels x the tile), landing as [octet][voxel][8],
-// and g's tile is one copy, [o-octet][voxel][8]; both are the canonical
-// MN-major layout (8 voxels x 8 channels per 128-byte core matrix, 128 bytes
-// apart along K = voxels, 2048 bytes apart along M or N), so the MMA reads
-// them as they land.  The 128 x cout FP32 accumulator stays in TMEM over the
-// CTA's voxel range and is written once as the CTA's partial sum; a second
-// kernel adds the partials in a fixed order.
+// of the tap-major row space (27 x cin rows), columns o, K = the voxels, in
+// tiles of 128.  Both operands are MN-major as the channels-last tensors lie in
+// shared memory after a TMA copy: rows (voxels) of span channels, swizzled.
+// The FP32 accumulators stay in TMEM over the CTA's range of tiles and are
+// written once as its partial sums; a second kernel adds the partials in a
+// fixed order.
+//
+// What bounds it is L2 (every tap reads the input again: 1.8 GB for the
+// 16 -> 16 layer at 128^3) and the one thread that issues the copies (16
+// copies of 16-byte rows with a division each took 570 us for that layer).
+//  - Tap tiles (grids narrower than 128): a CTA takes 128 rows: 128 / span
+//    copies per tile, one per (tap, block of span channels), from a table.
+//  - Halo rows (a tile is one row of 128 voxels): one copy per tile and 16
+//    channels of the box (130 x 3 x 3) around it, 9 reads of the input
+//    instead of 27.  The nine (dz, dy) rows of the box are 130 rows of 32
+//    bytes apart, so for each dx one operand of M = 128 takes eight of them as
+//    its blocks of 16 channels; the ninth row's three dx, 32 bytes apart, are
+//    a fourth operand (its other five blocks read what follows and are not
+//    used).  A CTA takes two of the four operands of one block of 16 channels:
+//    dx 0 and 1, or dx 2 and the ninth row.
+// The split over ranges of tiles follows the tap tiles' count of CTAs on both
+// paths: the tensor cores truncate as they accumulate, so sums over other
+// ranges would differ by more (6e-5) than the gradients' own precision.
 
 namespace gbmg {
 
 namespace {
 
 constexpr int kWgStages = 3;
+constexpr unsigned kWgHaloBytes = 9u * 130u * 32u;
 
 struct WgSmemHeader {
   unsigned long long full[kWgStages];
@@ -729,23 +796,38 @@ struct WgSmemHeader {
   uint32_t tmem;
   int abort;
   int consumed;
+  int4 box[8];  // tap tiles: dx, dy, dz and channel block of every copy
 };
+
+// bytes of one stage's input (a multiple of 1024; on the halo path with room
+// for the unused blocks' reads) and gradient
+__host__ __device__ unsigned wg_a_bytes(const WgradArgs& a) {
+  return a.halo ? (kWgHaloBytes + 8u * 32u + 1023u) / 1024u * 1024u : 128u * 256u;
+}
+__host__ __device__ unsigned wg_b_bytes(const WgradArgs& a) { return (unsigned)a.cout * 256u; }
+
+__host__ __device__ uint32_t wg_tmem_cols(const WgradArgs& a) {
+  const int c = a.cout * (a.halo ? 2 : 1);
+  return c <= 32 ? 32u : (c <= 64 ? 64u : (c <= 128 ? 128u : (c <= 256 ? 256u : 512u)));
+}
 
 __global__ void __launch_bounds__(kConvThreads, 1)
     wgrad_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_g, WgradArgs a) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   WgSmemHeader& S = *reinterpret_cast<WgSmemHeader*>(smem_raw);
-  const unsigned a_bytes = 16u * 2048u;
-  const unsigned b_bytes = (unsigned)a.cout * 256u;
+  const unsigned a_bytes = wg_a_bytes(a), b_bytes = wg_b_bytes(a);
+  const int NS = a.stages;
   unsigned char* stage_a = smem_raw + 1024;
-  unsigned char* stage_b = stage_a + kWgStages * a_bytes;
+  unsigned char* stage_b = stage_a + NS * a_bytes;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int mb = blockIdx.x % a.nmblk, sp = blockIdx.x / a.nmblk;
   const int T = a.ntx * a.nty * a.ntz;
   const int t_lo = (int)((long long)T * sp / a.nsplit), t_hi = (int)((long long)T * (sp + 1) / a.nsplit);
-  const uint32_t tcols = a.cout <= 32 ? 32u : (a.cout <= 64 ? 64u : 128u);
+  const uint32_t tcols = wg_tmem_cols(a);
+  const int copies = a.halo ? 1 : 128 / a.span;  // input copies per stage
+  const int hu = mb >> 1, hh = mb & 1;           // halo path: the CTA's 16 channels and half of the operands
   if (threadIdx.x == 0) {
-    for (int i = 0; i < kWgStages; ++i) {
+    for (int i = 0; i < NS; ++i) {
       mbar_init(&S.full[i], 1);
       mbar_init(&S.empty[i], 1);
     }
@@ -754,85 +836,146 @@ __global__ void __launch_bounds__(kConvThreads, 1)
     S.consumed = 0;
     mbar_init_fence();
   }
+  if (!a.halo && threadIdx.x >= 32 && threadIdx.x < 40) {
+    const int blocks = a.cin / a.span;
+    int R = mb * copies + (int)threadIdx.x - 32;
+    if (R >= 27 * blocks) R = 27 * blocks - 1;  // padding rows: any valid block (their sums are not used)
+    const int tap = R / blocks;
+    S.box[threadIdx.x - 32] = make_int4(tap % 3 - 1, (tap / 3) % 3 - 1, tap / 9 - 1, R % blocks);
+  }
+  if (a.halo && warp >= 2) {
+    // the rows after a halo box are read into unused accumulator rows: finite
+    for (int s = 0; s < NS; ++s)
+      for (unsigned o = kWgHaloBytes + 4u * (threadIdx.x - 64); o < a_bytes; o += 4u * 128u)
+        *reinterpret_cast<uint32_t*>(stage_a + s * a_bytes + o) = 0u;
+  }
   if (warp == 1) tmem_alloc(&S.tmem, tcols);
   tc_fence_before();
+  fence_proxy_async();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = S.tmem;
   volatile int* abort = &S.abort;
-  const int octets = a.cin / 8;
   if (warp == 0) {
     if (lane == 0) {
-      int it = 0;
-      for (int t = t_lo; t < t_hi; ++t, ++it) {
-        const int st = it % kWgStages, n = it / kWgStages;
-        if (n > 0 && !mbar_wait_bounded(&S.empty[st], (n - 1) & 1, kConvLimitNs, abort)) {
-          atomicExch(a.err, 1);
-          *abort = 1;
-          break;
-        }
+      const unsigned x_bytes = a.halo ? kWgHaloBytes : a_bytes;
+      int it = 0, st = 0;
+      uint32_t ph = 1;
+      bool stop = false;
+      for (int t = t_lo; t < t_hi && !stop; ++t) {
         const int tx = t % a.ntx, r = t / a.ntx, ty = r % a.nty, tz = r / a.nty;
         const int x0 = tx * a.bx, y0 = ty * a.by, z0 = tz * a.bz;
-        fence_proxy_async();
-        mbar_expect_tx(&S.full[st], a_bytes + b_bytes);
-        for (int g = 0; g < 16; ++g) {
-          int R = mb * 16 + g;  // row octet in the tap-major row space
-          if (R >= 27 * octets) R = 27 * octets - 1;  // padding rows: any valid octet (their sums are not used)
-          const int tap = R / octets, ic = R % octets;
-          const int dz = tap / 9, dy = (tap / 3) % 3, dx = tap % 3;
-          tma_load_5d(stage_a + st * a_bytes + g * 2048, &map_x, 0, x0 + dx - 1, y0 + dy - 1, z0 + dz - 1, ic,
-                      &S.full[st]);
+        if (it >= NS && !mbar_wait_bounded(&S.empty[st], ph, kConvLimitNs, abort)) {
+          atomicExch(a.err, 1);
+          *abort = 1;
+          stop = true;
+          break;
+        }
+        mbar_expect_tx(&S.full[st], x_bytes + b_bytes);
+        unsigned char* A = stage_a + st * a_bytes;
+        if (a.halo) {
+          tma_load_5d(A, &map_x, 0, x0 - 1, y0 - 1, z0 - 1, hu, &S.full[st]);
+        } else {
+#pragma unroll 1
+          for (int g = 0; g < copies; ++g) {
+            const int4 c = S.box[g];
+            tma_load_5d(A + g * 256 * a.span, &map_x, 0, x0 + c.x, y0 + c.y, z0 + c.z, c.w, &S.full[st]);
+          }
         }
         tma_load_5d(stage_b + st * b_bytes, &map_g, 0, x0, y0, z0, 0, &S.full[st]);
+        ++it;
+        if (++st == NS) {
+          st = 0;
+          ph ^= 1u;
+        }
       }
       if (*abort) {
-        for (int j = S.consumed; j < it; ++j) mbar_wait_bounded(&S.full[j % kWgStages], (j / kWgStages) & 1, kConvLimitNs);
+        for (int j = S.consumed; j < it; ++j) mbar_wait_bounded(&S.full[j % NS], (j / NS) & 1, kConvLimitNs);
       }
     }
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16_f32(kConvTileM, a.cout, true);
-      int it = 0;
+      // input: eight blocks of 16 channels 130 rows apart (halo), or blocks
+      // of span channels one after another; gradient: blocks of gspan channels
+      const uint32_t xs = 2u * (uint32_t)(a.halo ? 16 : a.span), gs = 2u * (uint32_t)a.gspan;
+      const uint64_t adesc = smem_desc_mn_swizzled(stage_a, xs, a.halo ? 130u * 32u : 128u * xs);
+      const uint64_t adesc9 = smem_desc_mn_swizzled(stage_a, 32u, 32u);  // the ninth row's taps, one row apart
+      const uint64_t bdesc = smem_desc_mn_swizzled(stage_b, gs, 128u * gs);
+      const uint32_t ahi = (uint32_t)(adesc >> 32), ahi9 = (uint32_t)(adesc9 >> 32), bhi = (uint32_t)(bdesc >> 32);
+      int it = 0, st = 0;
+      uint32_t ph = 0;
       bool issued = false;
-      for (int t = t_lo; t < t_hi && !*abort; ++t, ++it) {
-        const int st = it % kWgStages;
-        if (!mbar_wait_bounded(&S.full[st], (it / kWgStages) & 1, kConvLimitNs, abort)) {
+      for (int t = t_lo; t < t_hi && !*abort; ++t) {
+        if (!mbar_wait_bounded(&S.full[st], ph, kConvLimitNs, abort)) {
           atomicExch(a.err, 1);
           *abort = 1;
           break;
         }
         S.consumed = it + 1;
         tc_fence_after();
-        const unsigned char* A = stage_a + st * a_bytes;
-        const unsigned char* Bm = stage_b + st * b_bytes;
-        for (int ks = 0; ks < 8; ++ks) {
-          const uint64_t ad = smem_desc_mnmajor(A + ks * 256, 128, 2048);
-          const uint64_t bd = smem_desc_mnmajor(Bm + ks * 256, 128, 2048);
-          tc_mma_f16(tmem, ad, bd, idesc, (t > t_lo || ks > 0) ? 1u : 0u);
+        const uint32_t alo = (uint32_t)adesc + (uint32_t)st * (a_bytes >> 4);
+        const uint32_t blo = (uint32_t)bdesc + (uint32_t)st * (b_bytes >> 4);
+        const uint32_t acc0 = t > t_lo ? 1u : 0u;
+        if (a.halo) {
+          // dx = 0 and 1 (half 0), or dx = 2 and the ninth row (half 1), in
+          // steps of 16 voxels, 32 units of 16 bytes
+          const uint32_t a0 = alo + (hh ? 4u : 0u);
+          const uint32_t a1 = hh ? (uint32_t)adesc9 + (uint32_t)st * (a_bytes >> 4) + 8u * 130u * 2u : alo + 2u;
+          const uint32_t a1hi = hh ? ahi9 : ahi;
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks) {
+            const uint32_t b = blo + (uint32_t)ks * gs;
+            const uint32_t acc = ks > 0 ? 1u : acc0;
+            tc_mma_f16_words(tmem, a0 + (uint32_t)(ks * 32), ahi, b, bhi, idesc, acc);
+            tc_mma_f16_words(tmem + (uint32_t)a.cout, a1 + (uint32_t)(ks * 32), a1hi, b, bhi, idesc, acc);
+          }
+        } else {
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks)
+            tc_mma_f16_words(tmem, alo + (uint32_t)ks * xs, ahi, blo + (uint32_t)ks * gs, bhi, idesc, ks > 0 ? 1u : acc0);
         }
         tc_commit(&S.empty[st]);
         issued = true;
+        ++it;
+        if (++st == NS) {
+          st = 0;
+          ph ^= 1u;
+        }
       }
       if (!*abort) tc_commit(&S.accf);
       else if (issued)
-        for (int j = (it > kWgStages ? it - kWgStages : 0); j < it; ++j)
-          mbar_wait_bounded(&S.empty[j % kWgStages], (j / kWgStages) & 1, kConvLimitNs);
+        for (int j = (it > NS ? it - NS : 0); j < it; ++j)
+          mbar_wait_bounded(&S.empty[j % NS], (j / NS) & 1, kConvLimitNs);
     }
   } else {
     const int q = warp & 3;
     int ok = 1;
-    if (lane == 0) ok = mbar_wait_bounded(&S.accf, 0, kConvLimitNs, abort) ? 1 : 0;
+    if (lane == 0) ok = mbar_wait_bounded(&S.accf, 0, 4 * kConvLimitNs, abort) ? 1 : 0;
     ok = __shfl_sync(0xffffffffu, ok, 0);
     if (ok) {
       __syncwarp();
       tc_fence_after();
-      const int row = mb * 128 + 32 * q + lane;
-      float* dst = a.partial + ((size_t)sp * a.nmblk * 128 + row) * a.cout;
-      for (int c0 = 0; c0 < a.cout; c0 += 16) {
-        float v[16];
-        tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)c0, v);
+      const int m = 32 * q + lane;
+      const int nacc = a.halo ? 2 : 1;
+      for (int j = 0; j < nacc; ++j) {
+        int row = mb * 128 + m;
+        bool use = true;
+        if (a.halo) {  // operand dx: block m / 16 is (dz, dy); operand 3: the ninth's dx
+          const int k = 2 * hh + j, blk = m >> 4;
+          const int tap = k < 3 ? 3 * blk + k : 24 + blk;
+          row = tap * a.cin + 16 * hu + (m & 15);
+          use = k < 3 || blk < 3;
+        }
+        float* dst = a.partial + ((size_t)sp * a.rows + row) * a.cout;
+        for (int c0 = 0; c0 < a.cout; c0 += 16) {
+          float v[16];
+          tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(j * a.cout + c0), v);
+          if (!use) continue;
+          float4* o = reinterpret_cast<float4*>(dst + c0);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) dst[c0 + i] = v[i];
+          for (int i = 0; i < 4; ++i) o[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        }
       }
     } else if (lane == 0) {
       if (!*abort) atomicExch(a.err, 1);
@@ -845,93 +988,144 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   if (warp == 1) tmem_dealloc(tmem, tcols);
 }
 
-// dW[o][i][tap] (+)= sum over splits of partial[split][tap * cin_pad + i][o],
-// in split order; i < cin (the real input channels).
+// dW[o][i][tap] = sum over splits of partial[split][tap * cin_pad + i][o], in
+// split order; i < cin (the real input channels); neighbouring threads take
+// neighbouring o, the partials' fastest index.
 __global__ void wgrad_reduce_kernel(const float* __restrict__ partial, int nsplit, int rows, int cin_pad, int cin,
                                     int cout, float* __restrict__ dw) {
-  const long long n = (long long)cout * cin * 27;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const int tap = (int)(e % 27);
-    const long long r = e / 27;
-    const int i = (int)(r % cin), o = (int)(r / cin);
-    const size_t row = (size_t)tap * cin_pad + i;
+  const int n = 27 * cin * cout;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const int r = e / cout, o = e - r * cout;
+    const int tap = r / cin, i = r - tap * cin;
+    const float* p = partial + ((size_t)tap * cin_pad + i) * cout + o;
     float acc = 0.0f;
-    for (int s = 0; s < nsplit; ++s) acc += partial[((size_t)s * rows + row) * cout + o];
-    dw[e] = acc;
+#pragma unroll 8
+    for (int s = 0; s < nsplit; ++s) acc += p[(size_t)s * rows * cout];
+    dw[((size_t)o * cin + i) * 27 + tap] = acc;
+  }
+}
+
+// A block's threads of the per-channel sums below: every thread keeps one
+// group of 8 channels, `lanes` voxels at a time.
+struct ChannelLanes {
+  int G, lanes, g, l;
+  bool on;
+};
+__device__ __forceinline__ ChannelLanes channel_lanes(int c) {
+  ChannelLanes x;
+  x.G = c / 8;
+  x.lanes = blockDim.x / x.G;
+  x.l = threadIdx.x / x.G;
+  x.g = threadIdx.x - x.l * x.G;
+  x.on = x.l < x.lanes;
+  return x;
+}
+// The threads' 8 sums each into out[c], in a fixed order.
+__device__ __forceinline__ void channel_reduce(const ChannelLanes& x, const float* acc, int c, float (*sh)[9], float* out) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) sh[threadIdx.x][i] = acc[i];
+  __syncthreads();
+  for (int k = threadIdx.x; k < c; k += blockDim.x) {
+    float s = 0.0f;
+    for (int l = 0; l < x.lanes; ++l) s += sh[l * x.G + (k >> 3)][k & 7];
+    out[k] = s;
   }
 }
 
 // Per-block partial sums over voxels of g[v][o] (bias gradient), one row of
 // partials per block; then a fixed-order reduction.
-__global__ void channel_sum_kernel(const __nv_bfloat16* __restrict__ g, int c, long long V, float* __restrict__ part) {
-  extern __shared__ float sh[];
-  for (int o = threadIdx.x; o < c; o += blockDim.x) sh[o] = 0.0f;
-  __syncthreads();
-  const long long per = (V + gridDim.x - 1) / gridDim.x;
-  const long long lo = blockIdx.x * per, hi = min(V, lo + per);
-  // each thread owns one channel and a stride of voxels
-  const int lanes = blockDim.x / c;
-  const int o = threadIdx.x % c, l = threadIdx.x / c;
-  float acc = 0.0f;
-  if (l < lanes)
-    for (long long v = lo + l; v < hi; v += lanes) acc += __bfloat162float(g[v * c + o]);
-  if (l < lanes) atomicAdd(&sh[o], acc);  // within the block only
-  __syncthreads();
-  for (int k = threadIdx.x; k < c; k += blockDim.x) part[(size_t)blockIdx.x * c + k] = sh[k];
+__global__ void __launch_bounds__(256) channel_sum_kernel(const __nv_bfloat16* __restrict__ g, int c, long long V,
+                                                          float* __restrict__ part) {
+  __shared__ float sh[256][9];
+  const ChannelLanes x = channel_lanes(c);
+  float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  if (x.on) {
+    const long long step = (long long)gridDim.x * x.lanes;
+#pragma unroll 4
+    for (long long v = (long long)blockIdx.x * x.lanes + x.l; v < V; v += step) {
+      float f[8];
+      unpack8(load8(g + v * c + 8 * x.g), f);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i] += f[i];
+    }
+  }
+  channel_reduce(x, acc, c, sh, part + (size_t)blockIdx.x * c);
 }
 
-__global__ void partial_rows_sum_kernel(const float* __restrict__ part, int nrows, int c, float* __restrict__ out) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < c; k += gridDim.x * blockDim.x) {
-    float acc = 0.0f;
-    for (int r = 0; r < nrows; ++r) acc += part[(size_t)r * c + k];
-    out[k] = acc;
+// out[k] = sum of part[r][k] over the rows: 32 columns per block, 8 rows at a
+// time.
+__global__ void __launch_bounds__(256) partial_rows_sum_kernel(const float* __restrict__ part, int nrows, int c,
+                                                               float* __restrict__ out) {
+  __shared__ float sh[8][32];
+  const int k = blockIdx.x * 32 + (threadIdx.x & 31), l = threadIdx.x >> 5;
+  float acc = 0.0f;
+  if (k < c) {
+#pragma unroll 8
+    for (int r = l; r < nrows; r += 8) acc += part[(size_t)r * c + k];
+  }
+  sh[l][threadIdx.x & 31] = acc;
+  __syncthreads();
+  if (l == 0 && k < c) {
+    float s = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s += sh[i][threadIdx.x];
+    out[k] = s;
   }
 }
 
 // Head backward.  g_pred (FP32, dL/dpred), act = input channel 1 > 0:
 // gz[v][i] = (top[v][i] > 0) w[i] g act (BF16), and per-block partial sums
 // of g act top[v][i] (head weights) and g act (head bias).
-__global__ void head_backward_kernel(const float* __restrict__ gp, const __nv_bfloat16* __restrict__ x0,
-                                     const __nv_bfloat16* __restrict__ top, int c, const float* __restrict__ w,
-                                     long long V, __nv_bfloat16* __restrict__ gz, float* __restrict__ part) {
-  extern __shared__ float sh[];  // [c + 1]
-  for (int k = threadIdx.x; k <= c; k += blockDim.x) sh[k] = 0.0f;
-  __syncthreads();
-  float acc_b = 0.0f;
-  float acc_w[64];
-  for (int i = 0; i < c && i < 64; ++i) acc_w[i] = 0.0f;
-  for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < V; v += (long long)gridDim.x * blockDim.x) {
-    const float g = __bfloat162float(x0[v * 16 + 1]) > 0.0f ? gp[v] : 0.0f;
-    acc_b += g;
-    for (int i = 0; i < c; ++i) {
-      const float t = __bfloat162float(top[v * c + i]);
-      acc_w[i] += g * t;
-      gz[v * c + i] = __float2bfloat16_rn(t > 0.0f ? w[i] * g : 0.0f);
+__global__ void __launch_bounds__(256)
+    head_backward_kernel(const float* __restrict__ gp, const __nv_bfloat16* __restrict__ x0,
+                         const __nv_bfloat16* __restrict__ top, int c, const float* __restrict__ w, long long V,
+                         __nv_bfloat16* __restrict__ gz, float* __restrict__ part) {
+  __shared__ float sh[256][9];
+  __shared__ float bias[256];
+  const ChannelLanes x = channel_lanes(c);
+  float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0}, acc_b = 0.0f;
+  if (x.on) {
+    float wv[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) wv[i] = w[8 * x.g + i];
+    const long long step = (long long)gridDim.x * x.lanes;
+#pragma unroll 2
+    for (long long v = (long long)blockIdx.x * x.lanes + x.l; v < V; v += step) {
+      const uint32_t m = *reinterpret_cast<const uint32_t*>(x0 + v * 16);  // channels 0 and 1
+      const float g = __uint_as_float(m & 0xffff0000u) > 0.0f ? gp[v] : 0.0f;
+      acc_b += g;
+      float t[8], o[8];
+      unpack8(load8(top + v * c + 8 * x.g), t);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        acc[i] += g * t[i];
+        o[i] = t[i] > 0.0f ? wv[i] * g : 0.0f;
+      }
+      *reinterpret_cast<uint4*>(gz + v * c + 8 * x.g) = pack8(o);
     }
   }
-  for (int i = 0; i < c; ++i) atomicAdd(&sh[i], acc_w[i]);
-  atomicAdd(&sh[c], acc_b);
-  __syncthreads();
-  for (int k = threadIdx.x; k <= c; k += blockDim.x) part[(size_t)blockIdx.x * (c + 1) + k] = sh[k];
+  bias[threadIdx.x] = x.on && x.g == 0 ? acc_b : 0.0f;
+  channel_reduce(x, acc, c, sh, part + (size_t)blockIdx.x * (c + 1));
+  if (threadIdx.x == 0) {
+    float s = 0.0f;
+    for (int l = 0; l < x.lanes; ++l) s += bias[l * x.G];
+    part[(size_t)blockIdx.x * (c + 1) + c] = s;
+  }
 }
 
 // Gradient through nearest upsampling: dst[v][i] = sum over the 8 children of
 // src[child][so + i] (src at twice the size), FP32 sum rounded to BF16.
 __global__ void upsample_backward_kernel(const __nv_bfloat16* __restrict__ src, int ss, int so, int W, int H, int D,
                                          int c, __nv_bfloat16* __restrict__ dst) {
-  const long long n = (long long)W * H * D * c;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(e % c);
-    const long long v = e / c;
-    const int x = (int)(v % W), y = (int)((v / W) % H), z = (int)(v / ((long long)W * H));
-    float acc = 0.0f;
-    for (int dz = 0; dz < 2; ++dz)
-      for (int dy = 0; dy < 2; ++dy)
-        for (int dx = 0; dx < 2; ++dx) {
-          const long long vs = ((long long)(2 * z + dz) * (2 * H) + (2 * y + dy)) * (2 * W) + (2 * x + dx);
-          acc += __bfloat162float(src[vs * ss + so + i]);
-        }
-    dst[e] = __float2bfloat16_rn(acc);
+  const int G = c / 8;
+  for (int row = blockIdx.x; row < H * D; row += gridDim.x) {
+    const int z = row / H, y = row - z * H;
+    for (int e = threadIdx.x; e < W * G; e += blockDim.x) {
+      const int x = e / G, g = e - x * G;
+      float acc[8];
+      child_sum8(src, ss, so + 8 * g, W, H, x, y, z, acc);
+      *reinterpret_cast<uint4*>(dst + ((long long)row * W + x) * c + 8 * g) = pack8(acc);
+    }
   }
 }
 
@@ -942,15 +1136,21 @@ __global__ void skip_pool_combine_kernel(const __nv_bfloat16* __restrict__ skip,
                                          const __nv_bfloat16* __restrict__ act, int as,
                                          const __nv_bfloat16* __restrict__ gpool, int W, int H, int D, int c,
                                          __nv_bfloat16* __restrict__ gz) {
-  const long long n = (long long)W * H * D * c;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(e % c);
-    const long long v = e / c;
-    const int x = (int)(v % W), y = (int)((v / W) % H), z = (int)(v / ((long long)W * H));
-    const long long vp = ((long long)(z >> 1) * (H / 2) + (y >> 1)) * (W / 2) + (x >> 1);
-    const float a = __bfloat162float(act[v * as + i]);
-    const float gpv = a > 0.0f ? 0.125f * __bfloat162float(gpool[vp * c + i]) : 0.0f;
-    gz[e] = __float2bfloat16_rn(__bfloat162float(skip[v * ss + i]) + gpv);
+  const int G = c / 8;
+  for (int row = blockIdx.x; row < H * D; row += gridDim.x) {
+    const int z = row / H, y = row - z * H;
+    const long long prow = ((long long)(z >> 1) * (H / 2) + (y >> 1)) * (W / 2);
+    for (int e = threadIdx.x; e < W * G; e += blockDim.x) {
+      const int x = e / G, g = e - x * G;
+      const long long v = (long long)row * W + x;
+      float a[8], p[8], k[8];
+      unpack8(load8(act + v * as + 8 * g), a);
+      unpack8(load8(gpool + (prow + (x >> 1)) * c + 8 * g), p);
+      unpack8(load8(skip + v * ss + 8 * g), k);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) k[i] += a[i] > 0.0f ? 0.125f * p[i] : 0.0f;
+      *reinterpret_cast<uint4*>(gz + v * c + 8 * g) = pack8(k);
+    }
   }
 }
 
@@ -1023,7 +1223,36 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, 
 
 }  // namespace
 
-size_t wgrad_smem_bytes(int cout) { return 1024 + (size_t)kWgStages * (16 * 2048 + (size_t)cout * 256); }
+size_t wgrad_smem_bytes(const WgradArgs& a) {
+  return 1024 + (size_t)a.stages * (wg_a_bytes(a) + wg_b_bytes(a));
+}
+
+void wgrad_plan(WgradArgs& a) {
+  auto span_of = [](int c) { return c % 64 == 0 ? 64 : (c % 32 == 0 ? 32 : 16); };
+  conv_tile_box(a.W, a.H, a.D, kConvTileM, &a.bx, &a.by, &a.bz);
+  a.ntx = (a.W + a.bx - 1) / a.bx;
+  a.nty = (a.H + a.by - 1) / a.by;
+  a.ntz = (a.D + a.bz - 1) / a.bz;
+  a.gspan = span_of(a.cout);
+  a.halo = a.bx == 128 ? 1 : 0;
+  a.span = a.halo ? 16 : span_of(a.cin);
+  const int blocks = (27 * a.cin + 127) / 128;
+  a.nmblk = a.halo ? 2 * (a.cin / 16) : blocks;
+  a.rows = a.halo ? 27 * a.cin : blocks * 128;
+  const int T = a.ntx * a.nty * a.ntz;
+  int ns = 2 * device_sms() / blocks;
+  if (ns < 1) ns = 1;
+  a.nsplit = ns > T ? T : ns;
+  // halo stages are 42 KB: a third one only while a CTA has its SM for itself
+  a.stages = a.halo && a.nmblk * a.nsplit > device_sms() ? 2 : kWgStages;
+}
+
+bool make_wgrad_maps(CUtensorMap* mx, CUtensorMap* mg, const __nv_bfloat16* x, const __nv_bfloat16* g,
+                     const WgradArgs& a) {
+  const bool okx = a.halo ? make_conv_input_map(mx, x, a.W, a.H, a.D, a.cin, 16, 130, 3, 3, 1)
+                          : make_conv_input_map(mx, x, a.W, a.H, a.D, a.cin, a.span, a.bx, a.by, a.bz, 1);
+  return okx && make_conv_input_map(mg, g, a.W, a.H, a.D, a.cout, a.gspan, a.bx, a.by, a.bz, a.cout / a.gspan);
+}
 
 cudaError_t init_wgrad_kernel(size_t smem_bytes) {
   return cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
@@ -1031,7 +1260,7 @@ cudaError_t init_wgrad_kernel(size_t smem_bytes) {
 
 cudaError_t launch_wgrad(const CUtensorMap& mx, const CUtensorMap& mg, const WgradArgs& a, cudaStream_t s) {
   count_launch();
-  wgrad_kernel<<<a.nmblk * a.nsplit, kConvThreads, wgrad_smem_bytes(a.cout), s>>>(mx, mg, a);
+  wgrad_kernel<<<a.nmblk * a.nsplit, kConvThreads, wgrad_smem_bytes(a), s>>>(mx, mg, a);
   return cudaGetLastError();
 }
 
@@ -1045,8 +1274,8 @@ cudaError_t launch_wgrad_reduce(const float* partial, int nsplit, int rows, int 
 cudaError_t launch_bias_grad(const __nv_bfloat16* g, int c, long long V, float* part, int nblocks, float* db,
                              cudaStream_t s) {
   count_launch(2);
-  channel_sum_kernel<<<nblocks, 256, sizeof(float) * c, s>>>(g, c, V, part);
-  partial_rows_sum_kernel<<<1, 256, 0, s>>>(part, nblocks, c, db);
+  channel_sum_kernel<<<nblocks, 256, 0, s>>>(g, c, V, part);
+  partial_rows_sum_kernel<<<(c + 31) / 32, 256, 0, s>>>(part, nblocks, c, db);
   return cudaGetLastError();
 }
 
@@ -1054,15 +1283,15 @@ cudaError_t launch_head_backward(const float* gp, const __nv_bfloat16* x0, const
                                  const float* w, long long V, __nv_bfloat16* gz, float* part, int nblocks, float* dwb,
                                  cudaStream_t s) {
   count_launch(2);
-  head_backward_kernel<<<nblocks, 256, sizeof(float) * (c + 1), s>>>(gp, x0, top, c, w, V, gz, part);
-  partial_rows_sum_kernel<<<1, 256, 0, s>>>(part, nblocks, c + 1, dwb);
+  head_backward_kernel<<<nblocks, 256, 0, s>>>(gp, x0, top, c, w, V, gz, part);
+  partial_rows_sum_kernel<<<(c + 32) / 32, 256, 0, s>>>(part, nblocks, c + 1, dwb);
   return cudaGetLastError();
 }
 
 cudaError_t launch_upsample_backward(const __nv_bfloat16* src, int ss, int so, int W, int H, int D, int c,
                                      __nv_bfloat16* dst, cudaStream_t s) {
   count_launch();
-  upsample_backward_kernel<<<ew_grid((long long)W * H * D * c), 256, 0, s>>>(src, ss, so, W, H, D, c, dst);
+  upsample_backward_kernel<<<row_grid((long long)H * D), 256, 0, s>>>(src, ss, so, W, H, D, c, dst);
   return cudaGetLastError();
 }
 
@@ -1070,7 +1299,7 @@ cudaError_t launch_skip_pool_combine(const __nv_bfloat16* skip, int ss, const __
                                      const __nv_bfloat16* gpool, int W, int H, int D, int c, __nv_bfloat16* gz,
                                      cudaStream_t s) {
   count_launch();
-  skip_pool_combine_kernel<<<ew_grid((long long)W * H * D * c), 256, 0, s>>>(skip, ss, act, as, gpool, W, H, D, c, gz);
+  skip_pool_combine_kernel<<<row_grid((long long)H * D), 256, 0, s>>>(skip, ss, act, as, gpool, W, H, D, c, gz);
   return cudaGetLastError();
 }
 

@@ -193,13 +193,7 @@ mg_status setup_conv(mg_unet* N, Conv& C) {
 // mirrored weights, output `to` masked by `mask` where the layer's input is
 // a ReLU output) and the weight gradient's tensor maps and partition.
 mg_status setup_conv_backward(mg_unet* N, Conv& C, const Tensor* to, const Tensor* mask) {
-  int bx, by, bz;
-  conv_tile_box(C.in.W, C.in.H, C.in.D, kConvTileM, &bx, &by, &bz);
-  const int T = ((C.in.W + bx - 1) / bx) * ((C.in.H + by - 1) / by) * ((C.in.D + bz - 1) / bz);
   // weight gradient
-  if (!make_conv_input_map(&C.map_x1, C.in.p, C.in.W, C.in.H, C.in.D, C.cin_pad, 8, bx, by, bz, 1) ||
-      !make_conv_input_map(&C.map_g, C.gz.p, C.gz.W, C.gz.H, C.gz.D, C.cout, 8, bx, by, bz, C.cout / 8))
-    return ufail(N, MG_ERR_CUDA, "tensor map of a weight gradient was refused");
   WgradArgs& w = C.wg;
   std::memset(&w, 0, sizeof(w));
   w.W = C.in.W;
@@ -207,17 +201,9 @@ mg_status setup_conv_backward(mg_unet* N, Conv& C, const Tensor* to, const Tenso
   w.D = C.in.D;
   w.cin = C.cin_pad;
   w.cout = C.cout;
-  w.bx = bx;
-  w.by = by;
-  w.bz = bz;
-  w.ntx = (w.W + bx - 1) / bx;
-  w.nty = (w.H + by - 1) / by;
-  w.ntz = (w.D + bz - 1) / bz;
-  w.nmblk = (27 * C.cin_pad + 127) / 128;
-  int ns = (2 * device_sms()) / w.nmblk;
-  if (ns < 1) ns = 1;
-  if (ns > T) ns = T;
-  w.nsplit = ns;
+  wgrad_plan(w);
+  if (!make_wgrad_maps(&C.map_x1, &C.map_g, C.in.p, C.gz.p, w))
+    return ufail(N, MG_ERR_CUDA, "tensor map of a weight gradient was refused");
   w.err = N->err;
   if (!to) return MG_OK;
   // backward data: K = cout (the gradient's channels), N = cin_pad
@@ -254,7 +240,7 @@ mg_status finish_convs(mg_unet* N) {
   for (const Conv& C : N->convs) {
     most = C.smem > most ? C.smem : most;
     most = C.bsmem > most ? C.bsmem : most;
-    const size_t ws = wgrad_smem_bytes(C.cout);
+    const size_t ws = wgrad_smem_bytes(C.wg);
     most_w = ws > most_w ? ws : most_w;
   }
   UCK(N, init_conv_kernel(most));
@@ -311,7 +297,7 @@ mg_status conv_weight_grad(mg_unet* N, Conv& C) {
   WgradArgs a = C.wg;
   a.partial = N->wg_partial;
   UCK(N, launch_wgrad(C.map_x1, C.map_g, a, s));
-  UCK(N, launch_wgrad_reduce(N->wg_partial, a.nsplit, a.nmblk * 128, C.cin_pad, C.cin, C.cout, C.dw, s));
+  UCK(N, launch_wgrad_reduce(N->wg_partial, a.nsplit, a.rows, C.cin_pad, C.cin, C.cout, C.dw, s));
   UCK(N, launch_bias_grad(C.gz.p, C.cout, C.gz.voxels(), N->red_partial, N->red_blocks, C.db, s));
   return MG_OK;
 }
@@ -490,15 +476,15 @@ mg_status mg_unet_create(int levels, int base, int nx, int ny, int nz, void* cud
     const int l = C.level;
     const long long Vl = (long long)(nx >> l) * (ny >> l) * (nz >> l);
     o_gz[i] = R.take(sizeof(__nv_bfloat16) * (size_t)Vl * C.cout);
-    // weight-gradient partial sums (the partition of setup_conv_backward)
-    int bx, by, bz;
-    conv_tile_box(nx >> l, ny >> l, nz >> l, kConvTileM, &bx, &by, &bz);
-    const int T = (((nx >> l) + bx - 1) / bx) * (((ny >> l) + by - 1) / by) * (((nz >> l) + bz - 1) / bz);
-    const int nmblk = (27 * C.cin_pad + 127) / 128;
-    int ns = (2 * device_sms()) / nmblk;
-    if (ns < 1) ns = 1;
-    if (ns > T) ns = T;
-    const size_t wf = (size_t)ns * nmblk * 128 * C.cout;
+    // weight-gradient partial sums
+    WgradArgs wg = {};
+    wg.W = nx >> l;
+    wg.H = ny >> l;
+    wg.D = nz >> l;
+    wg.cin = C.cin_pad;
+    wg.cout = C.cout;
+    wgrad_plan(wg);
+    const size_t wf = (size_t)wg.nsplit * wg.rows * C.cout;
     wg_floats = wf > wg_floats ? wf : wg_floats;
   }
   const long long off_head = N->n_params;
@@ -512,7 +498,7 @@ mg_status mg_unet_create(int levels, int base, int nx, int ny, int nz, void* cud
   const size_t o_gpred = R.take(sizeof(float) * V0);
   const size_t o_target = R.take(sizeof(float) * V0);
   const size_t o_wgp = R.take(sizeof(float) * wg_floats);
-  N->red_blocks = 256;
+  N->red_blocks = 512;
   const size_t o_red = R.take(sizeof(float) * (size_t)N->red_blocks * (128 + 1));
   N->loss_blocks = 512;
   const size_t o_lp = R.take(sizeof(double) * (2 * (size_t)N->loss_blocks + 2));

@@ -83,24 +83,29 @@ int conv_grid(const ConvArgs& a, size_t smem_bytes);
 cudaError_t launch_pack_weights(const float* w, int cout, int cin, int cin_pad, bool backward, __nv_bfloat16* out,
                                 cudaStream_t s);
 
-// Weight gradient of one convolution (see kernels_unet.cu): CTA
-// (mblock, split) sums the voxel tiles [T split / nsplit, T (split+1) /
-// nsplit) into partial[split][mblock * 128 + row][o], rows (tap, i) of the
-// tap-major row space of cin (padded) input channels.
+// Weight gradient of one convolution (see kernels_unet.cu): rows (tap, i) of
+// the tap-major row space of cin (padded) input channels, split over ranges of
+// voxel tiles: partial[split][row][o], `rows` rows per split.
 struct WgradArgs {
   int W, H, D;
   int cin;     // padded input channels (the input tensor's channels), multiple of 16
   int cout;    // output channels, multiple of 16, <= 128
+  int span, gspan;  // channels per shared-memory row of the input and of the gradient
+  int halo;    // a tile is one row of 128 voxels whose input is copied with a halo
   int bx, by, bz, ntx, nty, ntz;
-  int nmblk;   // ceil(27 cin / 128)
+  int nmblk;   // CTAs per split: blocks of 128 rows, or on the halo path two per 16 channels
   int nsplit;  // <= the number of voxel tiles
+  int rows;
+  int stages;
   float* partial;
   int* err;
 };
-size_t wgrad_smem_bytes(int cout);
+// Everything but the pointers from W, H, D, cin and cout.
+void wgrad_plan(WgradArgs& a);
+bool make_wgrad_maps(CUtensorMap* mx, CUtensorMap* mg, const __nv_bfloat16* x, const __nv_bfloat16* g,
+                     const WgradArgs& a);
+size_t wgrad_smem_bytes(const WgradArgs& a);
 cudaError_t init_wgrad_kernel(size_t smem_bytes);
-// mx: the input tensor with box (8, bx, by, bz, 1); mg: the gradient tensor
-// (cout channels) with box (8, bx, by, bz, cout / 8)
 cudaError_t launch_wgrad(const CUtensorMap& mx, const CUtensorMap& mg, const WgradArgs& a, cudaStream_t s);
 cudaError_t launch_wgrad_reduce(const float* partial, int nsplit, int rows, int cin_pad, int cin, int cout, float* dw,
                                 cudaStream_t s);
