@@ -776,8 +776,9 @@ cudaError_t launch_tensor_to_natural(const __nv_bfloat16* t, int stride, int off
 //    bytes apart, so for each dx one operand of M = 128 takes eight of them as
 //    its blocks of 16 channels; the ninth row's three dx, 32 bytes apart, are
 //    a fourth operand (its other five blocks read what follows and are not
-//    used).  A CTA takes two of the four operands of one block of 16 channels:
-//    dx 0 and 1, or dx 2 and the ninth row.
+//    used).  A CTA takes the four operands of one block of 16 channels, or two
+//    of them (dx 0 and 1, or dx 2 and the ninth row) while that leaves every
+//    CTA an SM of its own.
 // The split over ranges of tiles follows the tap tiles' count of CTAs on both
 // paths: the tensor cores truncate as they accumulate, so sums over other
 // ranges would differ by more (6e-5) than the gradients' own precision.
@@ -807,7 +808,7 @@ __host__ __device__ unsigned wg_a_bytes(const WgradArgs& a) {
 __host__ __device__ unsigned wg_b_bytes(const WgradArgs& a) { return (unsigned)a.cout * 256u; }
 
 __host__ __device__ uint32_t wg_tmem_cols(const WgradArgs& a) {
-  const int c = a.cout * (a.halo ? 2 : 1);
+  const int c = a.cout * (a.halo ? 4 / a.halves : 1);
   return c <= 32 ? 32u : (c <= 64 ? 64u : (c <= 128 ? 128u : (c <= 256 ? 256u : 512u)));
 }
 
@@ -816,7 +817,7 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   WgSmemHeader& S = *reinterpret_cast<WgSmemHeader*>(smem_raw);
   const unsigned a_bytes = wg_a_bytes(a), b_bytes = wg_b_bytes(a);
-  const int NS = a.stages;
+  constexpr int NS = kWgStages;
   unsigned char* stage_a = smem_raw + 1024;
   unsigned char* stage_b = stage_a + NS * a_bytes;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -825,7 +826,8 @@ __global__ void __launch_bounds__(kConvThreads, 1)
   const int t_lo = (int)((long long)T * sp / a.nsplit), t_hi = (int)((long long)T * (sp + 1) / a.nsplit);
   const uint32_t tcols = wg_tmem_cols(a);
   const int copies = a.halo ? 1 : 128 / a.span;  // input copies per stage
-  const int hu = mb >> 1, hh = mb & 1;           // halo path: the CTA's 16 channels and half of the operands
+  // halo path: the CTA's 16 channels and its first and number of operands
+  const int hu = mb / a.halves, op0 = a.halves == 2 ? 2 * (mb & 1) : 0, nop = 4 / a.halves;
   if (threadIdx.x == 0) {
     for (int i = 0; i < NS; ++i) {
       mbar_init(&S.full[i], 1);
@@ -918,17 +920,30 @@ __global__ void __launch_bounds__(kConvThreads, 1)
         const uint32_t blo = (uint32_t)bdesc + (uint32_t)st * (b_bytes >> 4);
         const uint32_t acc0 = t > t_lo ? 1u : 0u;
         if (a.halo) {
-          // dx = 0 and 1 (half 0), or dx = 2 and the ninth row (half 1), in
-          // steps of 16 voxels, 32 units of 16 bytes
-          const uint32_t a0 = alo + (hh ? 4u : 0u);
-          const uint32_t a1 = hh ? (uint32_t)adesc9 + (uint32_t)st * (a_bytes >> 4) + 8u * 130u * 2u : alo + 2u;
-          const uint32_t a1hi = hh ? ahi9 : ahi;
+          // operand dx (0 .. 2) starts dx rows on, operand 3 at the ninth row;
+          // 16 voxels are 32 units of 16 bytes
+          const uint32_t ninth = (uint32_t)adesc9 + (uint32_t)st * (a_bytes >> 4) + 8u * 130u * 2u;
+          if (nop == 4) {
 #pragma unroll
-          for (int ks = 0; ks < 8; ++ks) {
-            const uint32_t b = blo + (uint32_t)ks * gs;
-            const uint32_t acc = ks > 0 ? 1u : acc0;
-            tc_mma_f16_words(tmem, a0 + (uint32_t)(ks * 32), ahi, b, bhi, idesc, acc);
-            tc_mma_f16_words(tmem + (uint32_t)a.cout, a1 + (uint32_t)(ks * 32), a1hi, b, bhi, idesc, acc);
+            for (int ks = 0; ks < 8; ++ks) {
+              const uint32_t b = blo + (uint32_t)ks * gs;
+              const uint32_t acc = ks > 0 ? 1u : acc0;
+              tc_mma_f16_words(tmem, alo + (uint32_t)(ks * 32), ahi, b, bhi, idesc, acc);
+              tc_mma_f16_words(tmem + (uint32_t)a.cout, alo + (uint32_t)(ks * 32 + 2), ahi, b, bhi, idesc, acc);
+              tc_mma_f16_words(tmem + 2u * (uint32_t)a.cout, alo + (uint32_t)(ks * 32 + 4), ahi, b, bhi, idesc, acc);
+              tc_mma_f16_words(tmem + 3u * (uint32_t)a.cout, ninth + (uint32_t)(ks * 32), ahi9, b, bhi, idesc, acc);
+            }
+          } else {
+            const uint32_t a0 = alo + 2u * (uint32_t)op0;
+            const uint32_t a1 = op0 == 2 ? ninth : alo + 2u;
+            const uint32_t a1hi = op0 == 2 ? ahi9 : ahi;
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks) {
+              const uint32_t b = blo + (uint32_t)ks * gs;
+              const uint32_t acc = ks > 0 ? 1u : acc0;
+              tc_mma_f16_words(tmem, a0 + (uint32_t)(ks * 32), ahi, b, bhi, idesc, acc);
+              tc_mma_f16_words(tmem + (uint32_t)a.cout, a1 + (uint32_t)(ks * 32), a1hi, b, bhi, idesc, acc);
+            }
           }
         } else {
 #pragma unroll
@@ -957,12 +972,12 @@ __global__ void __launch_bounds__(kConvThreads, 1)
       __syncwarp();
       tc_fence_after();
       const int m = 32 * q + lane;
-      const int nacc = a.halo ? 2 : 1;
+      const int nacc = a.halo ? nop : 1;
       for (int j = 0; j < nacc; ++j) {
         int row = mb * 128 + m;
         bool use = true;
         if (a.halo) {  // operand dx: block m / 16 is (dz, dy); operand 3: the ninth's dx
-          const int k = 2 * hh + j, blk = m >> 4;
+          const int k = op0 + j, blk = m >> 4;
           const int tap = k < 3 ? 3 * blk + k : 24 + blk;
           row = tap * a.cin + 16 * hu + (m & 15);
           use = k < 3 || blk < 3;
@@ -1224,7 +1239,7 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, 
 }  // namespace
 
 size_t wgrad_smem_bytes(const WgradArgs& a) {
-  return 1024 + (size_t)a.stages * (wg_a_bytes(a) + wg_b_bytes(a));
+  return 1024 + (size_t)kWgStages * (wg_a_bytes(a) + wg_b_bytes(a));
 }
 
 void wgrad_plan(WgradArgs& a) {
@@ -1237,14 +1252,13 @@ void wgrad_plan(WgradArgs& a) {
   a.halo = a.bx == 128 ? 1 : 0;
   a.span = a.halo ? 16 : span_of(a.cin);
   const int blocks = (27 * a.cin + 127) / 128;
-  a.nmblk = a.halo ? 2 * (a.cin / 16) : blocks;
   a.rows = a.halo ? 27 * a.cin : blocks * 128;
   const int T = a.ntx * a.nty * a.ntz;
   int ns = 2 * device_sms() / blocks;
   if (ns < 1) ns = 1;
   a.nsplit = ns > T ? T : ns;
-  // halo stages are 42 KB: a third one only while a CTA has its SM for itself
-  a.stages = a.halo && a.nmblk * a.nsplit > device_sms() ? 2 : kWgStages;
+  a.halves = a.halo && a.cin / 16 * 2 * a.nsplit <= device_sms() ? 2 : 1;
+  a.nmblk = a.halo ? a.halves * (a.cin / 16) : blocks;
 }
 
 bool make_wgrad_maps(CUtensorMap* mx, CUtensorMap* mg, const __nv_bfloat16* x, const __nv_bfloat16* g,

@@ -93,10 +93,10 @@ struct WgradArgs {
   int span, gspan;  // channels per shared-memory row of the input and of the gradient
   int halo;    // a tile is one row of 128 voxels whose input is copied with a halo
   int bx, by, bz, ntx, nty, ntz;
-  int nmblk;   // CTAs per split: blocks of 128 rows, or on the halo path two per 16 channels
+  int nmblk;   // CTAs per split: blocks of 128 rows, or on the halo path halves per 16 channels
   int nsplit;  // <= the number of voxel tiles
   int rows;
-  int stages;
+  int halves;  // halo path: CTAs per split and 16 channels
   float* partial;
   int* err;
 };
