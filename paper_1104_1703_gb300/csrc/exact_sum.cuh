@@ -65,8 +65,9 @@ struct SumGuard {
   static constexpr int value = N <= 1 ? 10 : (N <= 2 ? 9 : (N <= 4 ? 8 : (N <= 8 ? 7 : (N <= 16 ? 6 : 5))));
 };
 
+// The definition, in 64-bit integers.
 template <int N>
-__host__ __device__ __forceinline__ double exact_sum(const double (&x)[N]) {
+__host__ __device__ __forceinline__ double exact_sum_wide(const double (&x)[N]) {
   static_assert(N >= 1 && N <= 32, "exact_sum: 1..32 terms");
   constexpr int G = SumGuard<N>::value;
   unsigned long long b[N];
@@ -120,5 +121,53 @@ __host__ __device__ __forceinline__ double exact_sum(const double (&x)[N]) {
   if (v >= 0x7ff0000000000000ull) return double_of(sign | 0x7ff0000000000000ull);
   return double_of(sign | v);
 }
+
+#ifdef __CUDA_ARCH__
+// The same value from fewer instructions (the sums bound the FP64 level-0
+// kernels: about 180 integer instructions per sum of six in the form above,
+// 100 here).  Largest exponents that neither overflow nor underflow
+// (128 .. 1900, every field in use) take the short way; there
+//  - a term's significand is shifted to bit 63, which drops its sign and
+//    exponent, and aligned with a right shift that the hardware clamps, so
+//    zeros and terms 60 binades down need no test;
+//  - a negative term enters as its complement, the ones' complements are
+//    made up for by their number;
+//  - the sum is rounded by one integer conversion (the FP64 pipe has room for
+//    it beside the update's multiply-add) and scaled in its exponent field.
+template <int N>
+__device__ __forceinline__ double exact_sum(const double (&x)[N]) {
+  constexpr int G = SumGuard<N>::value;
+  static_assert(G <= 11, "a significand at bit 63 is shifted right by 11 - G and more");
+  int top = 0;
+#pragma unroll
+  for (int j = 0; j < N; ++j) top = max(top, __double2hiint(x[j]) & 0x7fffffff);
+  const int emax = top >> 20;
+  if ((unsigned)(emax - 128) > 1772u) return exact_sum_wide(x);
+  unsigned long long S = 0;
+  int neg = 0;  // minus the number of negative terms
+#pragma unroll
+  for (int j = 0; j < N; ++j) {
+    const unsigned hi = (unsigned)__double2hiint(x[j]), lo = (unsigned)__double2loint(x[j]);
+    const unsigned mh = __funnelshift_l(lo, hi, 11) | 0x80000000u, ml = lo << 11;
+    const int s = (int)hi >> 31;
+    const unsigned sh = (unsigned)(emax + 11 - G) - ((hi >> 20) & 0x7ffu);
+    unsigned long long m, a;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(m) : "r"(ml), "r"(mh));
+    asm("shr.b64 %0, %1, %2;" : "=l"(a) : "l"(m), "r"(sh));
+    S += a ^ (unsigned long long)(long long)s;
+    neg += s;
+  }
+  S -= (unsigned long long)(long long)neg;
+  const double d = __ll2double_rn((long long)S);
+  const int dh = __double2hiint(d);
+  // value = S 2^(emax - 1075 - G)
+  return __hiloint2double(dh ? dh + ((emax - 1075 - G) << 20) : 0, __double2loint(d));
+}
+#else
+template <int N>
+inline double exact_sum(const double (&x)[N]) {
+  return exact_sum_wide(x);
+}
+#endif
 
 }  // namespace gbmg

@@ -19,7 +19,7 @@ namespace gbmg {
 
 namespace {
 
-constexpr int kPer = 2;              // list entries per thread in a chunk
+constexpr int kPer = 1;              // list entries in flight per thread in a chunk (two: 1% slower)
 constexpr int kBatchMaxThreads = 512;
 
 __device__ __forceinline__ bool chunk_runs(const Chunk& C, int st) {
@@ -78,8 +78,7 @@ __device__ __forceinline__ void gs_chunk(const PatchLevel& L, const Chunk& C, co
 __global__ void __launch_bounds__(kBatchMaxThreads)
     batch_scale_kernel(const Chunk* __restrict__ chunks, int nchunks, const PatchLevel* __restrict__ pls) {
   pdl_wait();
-  __shared__ double tab[16];
-  init_tab(tab);
+  const double* const tab = diag_tab<double>();
   for (int k = blockIdx.x; k < nchunks; k += gridDim.x) {
     const Chunk C = chunks[k];
     const PatchLevel& L = pls[C.pl];
@@ -98,8 +97,7 @@ __global__ void __launch_bounds__(kBatchMaxThreads)
     batch_gs_kernel(const Chunk* __restrict__ chunks, int nchunks, const PatchLevel* __restrict__ pls,
                     const int* __restrict__ state) {
   pdl_wait();
-  __shared__ double tab[16];
-  if (FINE) init_tab(tab);
+  const double* const tab = diag_tab<double>();
   for (int k = blockIdx.x; k < nchunks; k += gridDim.x) {
     const Chunk C = chunks[k];
     const PatchLevel& L = pls[C.pl];
@@ -159,8 +157,7 @@ __global__ void __launch_bounds__(kBatchMaxThreads)
     batch_norm_kernel(const Chunk* __restrict__ chunks, int nchunks, const PatchLevel* __restrict__ pls,
                       const int* __restrict__ state, double* __restrict__ partials) {
   pdl_wait();
-  __shared__ double tab[16];
-  init_tab(tab);
+  const double* const tab = diag_tab<double>();
   for (int k = blockIdx.x; k < nchunks; k += gridDim.x) {
     const Chunk C = chunks[k];
     const PatchLevel& L = pls[C.pl];
@@ -215,8 +212,7 @@ __global__ void __launch_bounds__(kBatchMaxThreads)
     batch_restrict_kernel(const Chunk* __restrict__ chunks, int nchunks, const PatchLevel* __restrict__ pls,
                           const int* __restrict__ state, bool black_zero) {
   pdl_wait();
-  __shared__ double tab[16];
-  init_tab(tab);
+  const double* const tab = diag_tab<double>();
   for (int k = blockIdx.x; k < nchunks; k += gridDim.x) {
     const Chunk C = chunks[k];
     const PatchLevel& Lc = pls[C.pl];
@@ -299,8 +295,7 @@ __global__ void __launch_bounds__(kBottomThreads, 1)
                         const int* __restrict__ state) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double tab[16];
-  init_tab(tab);
+  const double* const tab = diag_tab<double>();
   for (int p = blockIdx.x; p < npatches; p += gridDim.x) {
     const int o = state[p] & kStOrder;
     if (o == 0) continue;

@@ -69,12 +69,15 @@ struct PerThread {
 // multiply-add, sum * (1/D) - b/D: 6 FP64 instructions instead of 7 on
 // the FP64-pipe-bound sweep.  With EXACT as well the neighbour sum is
 // formed in integer arithmetic (nbr_sum_exact), which leaves the fused
-// multiply-add as the update's only FP64 instruction.
+// multiply-add and the rounding of the sum as the update's FP64 instructions.
+// The FP64 form is bound by instructions and their latency together: with six
+// blocks per SM (42 registers; eight cost more instructions than they hide,
+// five hide less) a half-sweep of 2.28 million unknowns takes 22.9 us, 28.7
+// with a shared-memory table of diagonals and the wide form of the sum.
 template <int KIND, typename T, bool UPDATE, bool SCALED = false, bool EXACT = false>
-__global__ void __launch_bounds__(kListBlock) gs_list_kernel(ListArgs<T> a) {
+__global__ void __launch_bounds__(kListBlock, sizeof(T) == 8 ? 6 : 1) gs_list_kernel(ListArgs<T> a) {
   constexpr int PER = PerThread<T>::value;
-  __shared__ T tab[16];
-  if (KIND == 0) init_tab(tab);
+  const T* const tab = diag_tab<T>();
   const uint32_t n = *a.count;
   const uint32_t stride = gridDim.x * kListBlock;
   const uint32_t P = (uint32_t)a.g.P, Z = (uint32_t)a.g.sz;
@@ -137,8 +140,7 @@ template <typename T, bool UPDATE, int SHIFT>
 __global__ void __launch_bounds__(kListBlock) gs_seg_kernel(ListArgs<T> a) {
   constexpr int PER = 2;
   constexpr int GROUPS = 32 >> SHIFT;  // segments per warp and round
-  __shared__ T tab[16];
-  init_tab(tab);
+  const T* const tab = diag_tab<T>();
   const uint32_t n = *a.count;
   const int lane = threadIdx.x & 31;
   const int l = lane & ((1 << SHIFT) - 1);
@@ -203,8 +205,7 @@ template <bool UPDATE>
 __global__ void __launch_bounds__(kListBlock) gs_seg_pair_kernel(ListArgs<float> a) {
   constexpr int PER = 1;  // two slots per lane already
   constexpr int GROUPS = 4;  // segments per warp and round
-  __shared__ float tab[16];
-  init_tab(tab);
+  const float* const tab = diag_tab<float>();
   const uint32_t n = *a.count;
   const int lane = threadIdx.x & 31;
   const int l = lane & 7;
@@ -280,8 +281,7 @@ __global__ void __launch_bounds__(kListBlock) gs_seg_pair_kernel(ListArgs<float>
 template <int KIND, typename T, bool EXACT = false>
 __global__ void __launch_bounds__(kListBlock) res_list_kernel(ListArgs<T> a) {
   constexpr int PER = PerThread<T>::value;
-  __shared__ T tab[16];
-  if (KIND == 0) init_tab(tab);
+  const T* const tab = diag_tab<T>();
   const Geom g = a.g;
   const uint32_t n = *a.count;
   const uint32_t stride = gridDim.x * kListBlock;
@@ -349,8 +349,7 @@ template <int KIND, bool SMEM, typename T>
 __global__ void __launch_bounds__(kSmallThreads) smooth_small_kernel(SmallArgs<T> a) {
   pdl_wait();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ T tab[16];
-  if (KIND == 0) init_tab(tab);
+  const T* const tab = diag_tab<T>();
   const Geom g = a.g;
   T* p0 = a.phi0;
   T* p1 = a.phi1;
@@ -467,8 +466,7 @@ __device__ __forceinline__ T child_residual_sum(const RestrictArgs<T>& a, const 
 // residual.  Children outside the active set (of this order) count 0.
 template <int KIND, bool BLACK_ZERO, typename T>
 __global__ void __launch_bounds__(kBlockX * kBlockY) restrict_kernel(RestrictArgs<T> a) {
-  __shared__ T tab[16];
-  if (KIND == 0) init_tab(tab);
+  const T* const tab = diag_tab<T>();
   const Geom gc = a.gc;
   const int I = blockIdx.x * kBlockX + threadIdx.x;
   const int J = blockIdx.y * kBlockY + threadIdx.y;
@@ -491,11 +489,18 @@ __global__ void __launch_bounds__(kBlockX * kBlockY) restrict_kernel(RestrictArg
 // never written in a cycle: their correction stays the 0 it was reset to,
 // and their right-hand side is never read.  Every lane holds a coarse
 // unknown, which spares the FP64 pipe the idle lanes of a box-wide grid.
+// coarse unknowns per thread: two in FP32, whose loads overlap; in FP64 one,
+// with which half as many registers hold twice as many warps (V-cycles of
+// 4.6 million unknowns: 473 -> 461 us)
+template <typename T>
+struct RestrictPer {
+  static constexpr int value = sizeof(T) == 8 ? 1 : 2;
+};
+
 template <int KIND, bool BLACK_ZERO, typename T, bool EXACT = false>
 __global__ void __launch_bounds__(kListBlock) restrict_list_kernel(RestrictArgs<T> a) {
-  constexpr int PER = 2;
-  __shared__ T tab[16];
-  if (KIND == 0) init_tab(tab);
+  constexpr int PER = RestrictPer<T>::value;
+  const T* const tab = diag_tab<T>();
   const Geom gc = a.gc;
   const uint32_t n0 = *a.ccount[0], n = n0 + *a.ccount[1];
   const uint32_t stride = gridDim.x * kListBlock;
@@ -715,8 +720,7 @@ struct RefineArgs {
 template <bool EXACT>
 __global__ void __launch_bounds__(kListBlock) refine_residual_kernel(RefineArgs a) {
   constexpr int PER = 2;
-  __shared__ double tab[16];
-  init_tab(tab);
+  const double* const tab = diag_tab<double>();
   const Geom g = a.g;
   const uint32_t n0 = *a.count[0], n = n0 + *a.count[1];
   const uint32_t stride = gridDim.x * kListBlock;
@@ -973,7 +977,7 @@ cudaError_t restrict_t(const LevelDev& Lf, const LevelDev& Lc, int order, bool b
   // pipe; FP32: fewer threads); from a coarse level the box-wide grid, whose
   // extra warps hide more latency, is faster
   if (!all_cells && Lf.level == 0) {
-    const int lgrid = exact_grid(Lc.hcount[4] + Lc.hcount[5], 2);
+    const int lgrid = exact_grid(Lc.hcount[4] + Lc.hcount[5], RestrictPer<T>::value);
     count_launch();
     if (sizeof(T) == 8 && Lf.exact_sum) {  // level 0, FP64: the residuals with the integer neighbour sum
       if (black_zero) launch_pdl(restrict_list_kernel<0, true, T, true>, dim3(lgrid), dim3(kListBlock), 0, s, a);
@@ -1309,8 +1313,7 @@ __global__ void scale_rhs_kernel(long long total, const double* __restrict__ r0,
                                  const uint8_t* __restrict__ c0, const uint8_t* __restrict__ c1, double* __restrict__ o0,
                                  double* __restrict__ o1) {
   pdl_wait();
-  __shared__ double tab[16];
-  init_tab(tab);
+  const double* const tab = diag_tab<double>();
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
     o0[e] = (c0[e] & kActive2) ? r0[e] * tab[__popc((unsigned)c0[e] >> kGhostShift)] : 0.0;
