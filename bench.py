@@ -453,7 +453,7 @@ def roofline(st, n_active, precision, peaks, fp64_rate=None, pass_on=False, seg_
     ach = 13.0 * half / gs_s / 1e9
     if seg_on == 3:
         return {"bound": "hbm", "kernel": "gs_seg_pair_kernel (level-0 red/black Gauss-Seidel over 16-slot row "
-                                          "segments, two slots per thread, FP32 inner cycle)",
+                                          "segments, four slots per thread, FP32 inner cycle)",
                 "achieved": ach, "peak": hbm_peak, "unit": "GB/s", "frac": ach / hbm_peak,
                 "traffic": profiled_traffic("gs_seg_pair_fp32_level0_sphere_union_256.md"),
                 "launches": st["gs_n"], "avg_launch_us": gs_s * 1e6, "peak_source": src}

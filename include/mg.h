@@ -111,8 +111,9 @@ typedef enum { MG_MEM_HOST = 0, MG_MEM_DEVICE = 1 } mg_mem;
  *                  thread per slot of the row segments (8, 16 slots of one
  *                  colour's half-row) that hold an active cell, so that a
  *                  warp reads whole runs of every array; 3 = 16-slot
- *                  segments with two consecutive slots per thread (8-byte
- *                  loads); 0 = one thread per active cell of the colour's
+ *                  segments with four consecutive slots per thread
+ *                  (16-byte loads), in the restriction and prolongation of
+ *                  level 0 as well; 0 = one thread per active cell of the colour's
  *                  compact list.  The results are bit-identical.  (The FP64
  *                  sweeps always use the cell lists.)
  *  coarse_matrix   1 = solve the coarsest level, when it has at most 64

@@ -26,6 +26,8 @@
 // compact lists of the unknowns (built once per mask), where every lane holds
 // an unknown, and issue as few FP64 instructions as the operator allows.
 // Neighbour values come through L1/L2.
+#include <algorithm>
+
 #include "cycle_device.cuh"
 
 namespace gbmg {
@@ -192,84 +194,72 @@ __global__ void __launch_bounds__(kListBlock) gs_seg_kernel(ListArgs<T> a) {
   }
 }
 
-// The same sweep over 16-slot row segments with two consecutive slots per
-// lane (8-byte loads and stores): lane l of a group of 8 takes slots
-// q0 + 2l and q0 + 2l + 1.  The x-neighbour that is not in the lane's own
-// pair is the adjacent lane's (a shuffle within the group) or, for the
+// The same sweep over 16-slot row segments with two pairs of slots per lane
+// (16-byte loads and stores): lane l of a group of 4 takes slots q0 + 4l ..
+// q0 + 4l + 3.  A fine level larger than the L2 is bound by HBM (13 bytes per
+// update): at 512^3 with holes a half-sweep takes 135 us, 6.4 TB/s; with one
+// pair per lane 174, as many loads in flight but twice the instructions.  The x-neighbour that is not in the lane's own
+// four is the adjacent lane's (a shuffle within the group) or, for the
 // group's first or last lane, one extra load.  Per cell the sum and the
 // update are gs_list_kernel's, in the same order, so the results are
 // bit-identical.  Groups of a warp run their rounds together (the shuffles
 // need every lane); a group without a segment works on slot (0, 0, 0) of the
 // level, whose stencil lies inside the arrays, and stores nothing.
+constexpr int kPairUpdateBlocks = 6;  // per SM with UPDATE: 40 registers
+
 template <bool UPDATE>
-__global__ void __launch_bounds__(kListBlock) gs_seg_pair_kernel(ListArgs<float> a) {
-  constexpr int PER = 1;  // two slots per lane already
-  constexpr int GROUPS = 4;  // segments per warp and round
+__global__ void __launch_bounds__(kListBlock, UPDATE ? kPairUpdateBlocks : 8) gs_seg_pair_kernel(ListArgs<float> a) {
+  constexpr int GROUPS = 8;  // segments per warp and round
   const float* const tab = diag_tab<float>();
   const uint32_t n = *a.count;
   const int lane = threadIdx.x & 31;
-  const int l = lane & 7;
+  const int l = lane & 3;
   const uint32_t warp_group = ((blockIdx.x * kListBlock + threadIdx.x) >> 5) * GROUPS;
-  const uint32_t mine = (uint32_t)(lane >> 3);
-  const uint32_t ngroups = (gridDim.x * kListBlock >> 5) * GROUPS;
-  const uint32_t step = PER * ngroups;
+  const uint32_t mine = (uint32_t)(lane >> 2);
+  const uint32_t step = (gridDim.x * kListBlock >> 5) * GROUPS;
   const uint32_t P = (uint32_t)a.g.P, Z = (uint32_t)a.g.sz, safe = (uint32_t)a.g.off0;
-  uint32_t next[PER];
-#pragma unroll
-  for (int u = 0; u < PER; ++u) {
-    const uint32_t i = warp_group + mine + u * ngroups;
-    next[u] = i < n ? a.list[i] : 0u;
-  }
+  uint32_t next = warp_group + mine < n ? a.list[warp_group + mine] : 0u;
+  auto quad = [](const float* p) { return *reinterpret_cast<const float4*>(p); };
   pdl_wait();
   for (uint32_t wb = warp_group; wb < n; wb += step) {
-    uint32_t cur[PER];
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      cur[u] = next[u];
-      const uint32_t i = wb + step + mine + u * ngroups;
-      next[u] = i < n ? a.list[i] : 0u;
-    }
-    uint32_t at[PER];
-    bool ok[PER], plus[PER];
-    float2 oh[PER], ym[PER], yp[PER], zm[PER], zp[PER], bb[PER];
-    float edge[PER];
-    uint16_t cd[PER];
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      const uint32_t e = cur[u];
-      ok[u] = wb + mine + u * ngroups < n && entry_ok(a.g, e & kListAt, 9);
-      plus[u] = ok[u] && (e & kListPlusX) != 0;
-      at[u] = (ok[u] ? (e & kListAt) : safe) + 2u * (uint32_t)l;
-      oh[u] = *reinterpret_cast<const float2*>(a.other + at[u]);
-      ym[u] = *reinterpret_cast<const float2*>(a.other + (at[u] - P));
-      yp[u] = *reinterpret_cast<const float2*>(a.other + (at[u] + P));
-      zm[u] = *reinterpret_cast<const float2*>(a.other + (at[u] - Z));
-      zp[u] = *reinterpret_cast<const float2*>(a.other + (at[u] + Z));
-      bb[u] = *reinterpret_cast<const float2*>(a.rhs + at[u]);
-      cd[u] = *reinterpret_cast<const uint16_t*>(a.code + at[u]);
-      edge[u] = 0.f;
-      if (plus[u] ? l == 7 : l == 0) edge[u] = a.other[plus[u] ? at[u] + 2u : at[u] - 1u];
-    }
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      const float up = __shfl_up_sync(0xffffffffu, oh[u].y, 1, 8);    // o[at - 1]
-      const float dn = __shfl_down_sync(0xffffffffu, oh[u].x, 1, 8);  // o[at + 2]
-      // x-neighbours of the pair's two cells: dx = +1 (plus) or -1
-      const float x0 = plus[u] ? oh[u].y : (l == 0 ? edge[u] : up);
-      const float x1 = plus[u] ? (l == 7 ? edge[u] : dn) : oh[u].x;
-      const float s0 = ((oh[u].x + x0) + (ym[u].x + yp[u].x)) + (zm[u].x + zp[u].x);
-      const float s1 = ((oh[u].y + x1) + (ym[u].y + yp[u].y)) + (zm[u].y + zp[u].y);
-      const unsigned c0 = cd[u] & 0xffu, c1 = cd[u] >> 8;
-      const bool a0 = (c0 & kActive2) != 0, a1 = (c1 & kActive2) != 0;
-      const float v0 = (s0 - bb[u].x) * tab[__popc(c0 >> kGhostShift)];
-      const float v1 = (s1 - bb[u].y) * tab[__popc(c1 >> kGhostShift)];
-      if (!ok[u]) continue;
-      *reinterpret_cast<float2*>(a.self + at[u]) = make_float2(a0 ? v0 : 0.f, a1 ? v1 : 0.f);
-      if (UPDATE && (a0 || a1)) {
-        double2 ph = *reinterpret_cast<const double2*>(a.phi64 + at[u]);
-        if (a0) ph.x += widen_f32(v0);
-        if (a1) ph.y += widen_f32(v1);
-        *reinterpret_cast<double2*>(a.phi64 + at[u]) = ph;
+    const uint32_t e = next;
+    next = wb + step + mine < n ? a.list[wb + step + mine] : 0u;
+    const bool ok = wb + mine < n && entry_ok(a.g, e & kListAt, 9);
+    const bool plus = ok && (e & kListPlusX) != 0;
+    const uint32_t at = (ok ? (e & kListAt) : safe) + 4u * (uint32_t)l;
+    const float4 o = quad(a.other + at), ym = quad(a.other + (at - P)), yp = quad(a.other + (at + P)),
+                 zm = quad(a.other + (at - Z)), zp = quad(a.other + (at + Z)), b = quad(a.rhs + at);
+    const unsigned cd = *reinterpret_cast<const uint32_t*>(a.code + at);
+    float edge = 0.f;
+    if (plus ? l == 3 : l == 0) edge = a.other[plus ? at + 4u : at - 1u];
+    const float lo = __shfl_up_sync(0xffffffffu, o.w, 1, 4);    // o[at - 1]
+    const float hi = __shfl_down_sync(0xffffffffu, o.x, 1, 4);  // o[at + 4]
+    // x-neighbours of the four cells: dx = +1 (plus) or -1
+    const float xl = l == 0 ? edge : lo, xh = l == 3 ? edge : hi;
+    auto update = [&](float c, float x, float m, float p, float u, float v, float r, unsigned code) {
+      const float w = ((((c + x) + (m + p)) + (u + v)) - r) * tab[__popc((code & 0xffu) >> kGhostShift)];
+      return (code & kActive2) ? w : 0.f;
+    };
+    const float4 w = make_float4(update(o.x, plus ? o.y : xl, ym.x, yp.x, zm.x, zp.x, b.x, cd),
+                                 update(o.y, plus ? o.z : o.x, ym.y, yp.y, zm.y, zp.y, b.y, cd >> 8),
+                                 update(o.z, plus ? o.w : o.y, ym.z, yp.z, zm.z, zp.z, b.z, cd >> 16),
+                                 update(o.w, plus ? xh : o.z, ym.w, yp.w, zm.w, zp.w, b.w, cd >> 24));
+    if (!ok) continue;
+    *reinterpret_cast<float4*>(a.self + at) = w;
+    if (UPDATE) {  // an inactive cell's w is 0, its Phi stays as it is
+      double2* const ph = reinterpret_cast<double2*>(a.phi64 + at);
+      const unsigned act = cd & (kActive2 * 0x01010101u);
+      if (act & 0xffffu) {
+        double2 v = ph[0];
+        if (act & 0xffu) v.x += widen_f32(w.x);
+        if (act & 0xff00u) v.y += widen_f32(w.y);
+        ph[0] = v;
+      }
+      if (act >> 16) {
+        double2 v = ph[1];
+        if (act & 0xff0000u) v.x += widen_f32(w.z);
+        if (act >> 24) v.y += widen_f32(w.w);
+        ph[1] = v;
       }
     }
   }
@@ -401,6 +391,7 @@ struct RestrictArgs {
   T* cphi[2];
   const uint32_t* clist[2];   // restrict_list_kernel: second-order unknowns of the coarse level
   const uint32_t* ccount[2];
+  const uint8_t* ccode[2];    // restrict_pair_kernel: codes of the coarse level
 };
 
 // What the mask fixes about the children of coarse cell (I, J, K): their
@@ -552,6 +543,109 @@ __global__ void __launch_bounds__(kListBlock) restrict_list_kernel(RestrictArgs<
   }
 }
 
+// K5 from level 0 of the mixed form's FP32 cycles, after a complete sweep
+// (only red children carry a residual), two coarse cells per thread: the
+// coarse cells I = 2Q and 2Q + 1 of a row, one of each colour, share slot Q
+// of their colour arrays, and their children lie at the fine slots 2Q and
+// 2Q + 1 of four fine rows.  So a thread reads 8-byte pairs, the twelve rows
+// of black values once for all four children rows, and consecutive lanes read
+// consecutive pairs.  (One coarse cell per thread reads every other slot of
+// the rows, each row once per child: 373 us at 512^3 with holes.)  The
+// threads walk the coarse level's red list; an entry of its black list is
+// taken only if its red partner is no unknown.  The sums have
+// restrict_list_kernel's order, so the results are the same bits.  The grid
+// is the blocks that are resident together, each thread's next list entry
+// loaded a round ahead, so that a round costs one memory latency (213 us;
+// a block per 256 entries: three latencies, 330 us).
+constexpr int kRestrictPairBlocks = 3;  // per SM: 80 registers hold a round's loads
+
+// the two coarse cells at slot atc
+__device__ __forceinline__ void restrict_pair(const RestrictArgs<float>& a, const float* tab, uint32_t atc) {
+  const Geom& gc = a.gc;
+  const Geom& gf = a.gf;
+  if (!entry_ok(gc, atc, 5)) return;
+  int Q, J, K;
+  gc.slot_of(atc, &Q, &J, &K);
+  const int red = (J ^ K) & 1;            // the colour of coarse cell 2Q
+  const bool up = 2 * K + 1 < gf.nz;      // the second plane of children lies in the box
+  const uint32_t P = (uint32_t)gf.P, Z = (uint32_t)gf.sz;
+  const uint32_t x00 = (uint32_t)gf.at(2 * Q, 2 * J, 2 * K);
+  auto pair = [](const float* p) { return *reinterpret_cast<const float2*>(p); };
+  const bool act0 = (a.ccode[red][atc] & kActive2) != 0, act1 = (a.ccode[red ^ 1][atc] & kActive2) != 0;
+  // black rows 2J - 1 .. 2J + 2 of planes 2K - 1 .. 2K + 2 (without the
+  // corners); of a second plane that is the box's halo only what the first
+  // plane's children need is read
+  const float2 zero = make_float2(0.f, 0.f);
+  float2 o[4][4], p[2][2], b[2][2];
+  float edge[2][2];
+  uint16_t code[2][2];
+#pragma unroll
+  for (int dk = 0; dk < 2; ++dk)
+#pragma unroll
+    for (int dj = 0; dj < 2; ++dj) {
+      const uint32_t x = x00 + (dj ? P : 0u) + (dk ? Z : 0u);
+      const bool in = dk == 0 || up;
+      code[dk][dj] = *reinterpret_cast<const uint16_t*>(a.code[0] + x);
+      o[1 + dk][1 + dj] = pair(a.phi[1] + x);
+      o[1 + dk][3 * dj] = in ? pair(a.phi[1] + (dj ? x + P : x - P)) : zero;
+      o[3 * dk][1 + dj] = in ? pair(a.phi[1] + (dk ? x + Z : x - Z)) : zero;
+      edge[dk][dj] = in ? a.phi[1][(dj ^ dk) ? x + 2u : x - 1u] : 0.f;
+      p[dk][dj] = in ? pair(a.phi[0] + x) : zero;
+      b[dk][dj] = in ? pair(a.rhs[0] + x) : zero;
+    }
+  float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+  for (int dk = 0; dk < 2; ++dk)
+#pragma unroll
+    for (int dj = 0; dj < 2; ++dj) {
+      const float2 c = o[1 + dk][1 + dj], ym = o[1 + dk][dj], yp = o[1 + dk][2 + dj], zm = o[dk][1 + dj],
+                   zp = o[2 + dk][1 + dj];
+      const unsigned c0 = code[dk][dj] & 0xffu, c1 = code[dk][dj] >> 8;
+      const float x0 = (dj ^ dk) ? c.y : edge[dk][dj], x1 = (dj ^ dk) ? edge[dk][dj] : c.x;
+      const float r0 = fmaf(-tab[8 + __popc(c0 >> kGhostShift)], p[dk][dj].x,
+                            ((c.x + x0) + (ym.x + yp.x)) + (zm.x + zp.x)) - b[dk][dj].x;
+      const float r1 = fmaf(-tab[8 + __popc(c1 >> kGhostShift)], p[dk][dj].y,
+                            ((c.y + x1) + (ym.y + yp.y)) + (zm.y + zp.y)) - b[dk][dj].y;
+      if (c0 & a.bit) s0 += r0;
+      if (c1 & a.bit) s1 += r1;
+    }
+  if (act0) {
+    a.crhs[red][atc] = -0.5f * s0;
+    a.cphi[red][atc] = 0.f;
+  }
+  if (act1) {
+    a.crhs[red ^ 1][atc] = -0.5f * s1;
+    a.cphi[red ^ 1][atc] = 0.f;
+  }
+}
+
+__global__ void __launch_bounds__(kListBlock, kRestrictPairBlocks) restrict_pair_kernel(RestrictArgs<float> a) {
+  const float* const tab = diag_tab<float>();
+  const uint32_t n0 = *a.ccount[0], n1 = *a.ccount[1];
+  const uint32_t first = blockIdx.x * kListBlock + threadIdx.x, stride = gridDim.x * kListBlock;
+  uint32_t next = first < n0 ? a.clist[0][first] : 0u;
+  pdl_wait();
+  for (uint32_t i = first; i < n0; i += stride) {
+    const uint32_t atc = next & kListAt;
+    next = i + stride < n0 ? a.clist[0][i + stride] : 0u;
+    restrict_pair(a, tab, atc);
+  }
+  constexpr int N = 4;  // black entries looked at together
+  for (uint32_t i = first; i < n1; i += N * stride) {
+    uint32_t atc[N];
+    bool alone[N];
+#pragma unroll
+    for (int u = 0; u < N; ++u) atc[u] = i + u * stride < n1 ? a.clist[1][i + u * stride] & kListAt : 0u;
+#pragma unroll
+    for (int u = 0; u < N; ++u) alone[u] = i + u * stride < n1 && !(a.ccode[0][atc[u]] & kActive2);
+#pragma unroll 1
+    for (int u = 0; u < N; ++u) {
+      const uint32_t at = u == 0 ? atc[0] : (u == 1 ? atc[1] : (u == 2 ? atc[2] : atc[3]));
+      if (u == 0 ? alone[0] : (u == 1 ? alone[1] : (u == 2 ? alone[2] : alone[3]))) restrict_pair(a, tab, at);
+    }
+  }
+}
+
 template <typename T>
 struct ProlongArgs {
   Geom gf, gc;
@@ -618,6 +712,97 @@ __global__ void __launch_bounds__(kListBlock) prolong_list_kernel(ProlongArgs<T>
 #pragma unroll
     for (int u = 0; u < PER; ++u)
       if (ok[u]) a.phi[cc[u]][at[u]] = fma(w[u], T(1) / T(64), old[u]);
+  }
+}
+
+// K6 on the black unknowns of level 0 in the mixed form's FP32 cycles, over
+// the 16-slot row segments of the sweeps (gs_seg_pair_kernel): a lane takes
+// four consecutive slots of a row.  Their stencils share the four coarse rows
+// and, in each, five coarse cells, so four cells take 12 coarse loads and one
+// 16-byte update in place of 32 and four.  The list kernel is bound by its
+// instructions (an index computation and 9 loads per cell): 341 us at 512^3
+// with holes, this one 138 (two slots per lane 199; bytes at HBM rate 98).
+// Per cell the sum is p2_sum's, in its order.
+struct ProlongQuadArgs {
+  Geom gf, gc;
+  float* phi;             // black
+  const uint8_t* code;
+  const uint32_t* list;   // black segments
+  const uint32_t* count;
+  const float* cphi[2];
+};
+
+constexpr int kProlongQuadBlocks = 5;  // per SM: 46 registers
+
+__global__ void __launch_bounds__(kListBlock, kProlongQuadBlocks) prolong_quad_kernel(ProlongQuadArgs a) {
+  const Geom& gc = a.gc;
+  const uint32_t n = *a.count, step = gridDim.x * (kListBlock / 4);
+  const int lane = threadIdx.x & 3;
+  uint32_t i = blockIdx.x * (kListBlock / 4) + (threadIdx.x >> 2);
+  // the entries are fixed by the mask: the first is loaded before the wait on
+  // the previous kernel, each next one a round ahead
+  uint32_t next = i < n ? a.list[i] : 0u;
+  pdl_wait();
+  for (; i < n; i += step) {
+    const uint32_t e = next;
+    next = i + step < n ? a.list[i + step] : 0u;
+    uint32_t at = e & kListAt;
+    if (!entry_ok(a.gf, at, 6)) continue;
+    const bool plus = (e & kListPlusX) != 0;
+    int q, j, k;
+    a.gf.slot_of(at, &q, &j, &k);
+    at += 4u * (uint32_t)lane;
+    const unsigned cd = *reinterpret_cast<const uint32_t*>(a.code + at);
+    const float4 old = *reinterpret_cast<const float4*>(a.phi + at);
+    // parents 2p .. 2p + 3, at coarse slots p and p + 1 (q is a multiple of
+    // 16 and the coarse pitch one of at least half the fine row, so both lie
+    // in the row)
+    const int p = (q >> 1) + 2 * lane;
+    const int row = (int)gc.off0 + (k >> 1) * (int)gc.sz + (j >> 1) * gc.P + p;
+    const int dY = (j & 1) ? gc.P : -gc.P;
+    const int dZ = (k & 1) ? (int)gc.sz : -(int)gc.sz;
+    const bool odd = ((j >> 1) ^ (k >> 1)) & 1;  // the colour of parent 2p
+    const float* const A = a.cphi[odd ? 1 : 0];
+    const float* const B = a.cphi[odd ? 0 : 1];
+    // coarse cells 2p - 1 .. 2p + 2 (the fine cells are the left children) or
+    // 2p .. 2p + 4 (the right ones) of a coarse row, nearest first along x;
+    // the rows a step away in y or in z have the colours the other way round
+    struct Row {
+      float v[5];  // parents in v[1..4] (left) or v[0..3] (right)
+    };
+    auto coarse_row = [&](int off, bool flip) {
+      const float* const E = flip ? B : A;
+      const float* const O = flip ? A : B;
+      const int x = row + off;
+      const float2 ev = *reinterpret_cast<const float2*>(E + x), ov = *reinterpret_cast<const float2*>(O + x);
+      // 2p + 4 matters where 2p + 3 is a cell, so that slot p + 2 is in the
+      // row; the one corner before the first element of its array (of fine
+      // cell (0, 0, 0)) holds 0 and is not read
+      float f = 0.f;
+      if (plus ? p + 2 < gc.P : x >= 1) f = plus ? E[x + 2] : O[x - 1];
+      Row r;
+      r.v[0] = plus ? ev.x : f;
+      r.v[1] = plus ? ov.x : ev.x;
+      r.v[2] = plus ? ev.y : ov.x;
+      r.v[3] = plus ? ov.y : ev.y;
+      r.v[4] = plus ? f : ov.y;
+      return r;
+    };
+    const Row nn = coarse_row(0, false), y = coarse_row(dY, true), z = coarse_row(dZ, true),
+              yz = coarse_row(dY + dZ, false);
+    const float h = 1.f / 64.f;
+    const float was[4] = {old.x, old.y, old.z, old.w};
+    float out[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      // near and far values of the cell in the four rows
+      auto at_x = [&](const Row& r, bool far) { return plus != far ? r.v[u] : r.v[u + 1]; };
+      const float e1 = (at_x(nn, true) + at_x(y, false)) + at_x(z, false);
+      const float e2 = (at_x(yz, false) + at_x(z, true)) + at_x(y, true);
+      const float w = fmaf(3.f, e2, fmaf(27.f, at_x(nn, false), 9.f * e1)) + at_x(yz, true);
+      out[u] = (cd >> (8 * u)) & kActive2 ? fmaf(w, h, was[u]) : was[u];
+    }
+    if (cd & (kActive2 * 0x01010101u)) *reinterpret_cast<float4*>(a.phi + at) = make_float4(out[0], out[1], out[2], out[3]);
   }
 }
 
@@ -816,13 +1001,12 @@ int exact_grid(uint32_t n, int per) {
   return b < 1 ? 1 : (int)b;
 }
 
-// grid for n row segments of 2^shift slots (one lane per slot), at most
-// the blocks that stay resident together (8 per SM at 256 threads), which
-// then loop
-int seg_grid(uint32_t n, int shift) {
+// grid for n row segments of 2^shift lanes each, at most the blocks that stay
+// resident together (per_sm, 8 at 32 registers a thread), which then loop
+int seg_grid(uint32_t n, int shift, int per_sm = 8) {
   const long long groups_per_block = (long long)kListBlock >> shift;
   long long b = ((long long)n + groups_per_block - 1) / groups_per_block;
-  const long long cap = 8LL * device_sms();
+  const long long cap = (long long)per_sm * device_sms();
   if (b > cap) b = cap;
   return b < 1 ? 1 : (int)b;
 }
@@ -873,8 +1057,8 @@ cudaError_t half_sweep_seg(const LevelDev& L, int colour, bool update, cudaStrea
   a.phi64 = L.phi[colour];
   a.list = L.list[0][colour];
   a.count = L.count + colour;
-  if (SHIFT == 4 && L.seg_pairs) {  // 8 lanes per 16-slot segment: the grid of 8-slot segments
-    const int grid = seg_grid(L.hcount[colour], 3);
+  if (SHIFT == 4 && L.seg_pairs) {  // 4 lanes per 16-slot segment
+    const int grid = seg_grid(L.hcount[colour], 2, update ? kPairUpdateBlocks : 8);
     count_launch();
     if (update) launch_pdl(gs_seg_pair_kernel<true>, dim3(grid), dim3(kListBlock), 0, s, a);
     else launch_pdl(gs_seg_pair_kernel<false>, dim3(grid), dim3(kListBlock), 0, s, a);
@@ -976,6 +1160,15 @@ cudaError_t restrict_t(const LevelDev& Lf, const LevelDev& Lc, int order, bool b
   // over the coarse unknowns from level 0 (FP64: no idle lanes on the FP64
   // pipe; FP32: fewer threads); from a coarse level the box-wide grid, whose
   // extra warps hide more latency, is faster
+  if constexpr (sizeof(T) == 4) {
+    if (!all_cells && Lf.level == 0 && Lf.seg_pairs && black_zero) {
+      for (int c = 0; c < 2; ++c) a.ccode[c] = Lc.code[c];
+      count_launch();
+      const int pgrid = std::min(exact_grid(std::max(Lc.hcount[4], Lc.hcount[5]), 1), kRestrictPairBlocks * device_sms());
+      launch_pdl(restrict_pair_kernel, dim3(pgrid), dim3(kListBlock), 0, s, a);
+      return cudaGetLastError();
+    }
+  }
   if (!all_cells && Lf.level == 0) {
     const int lgrid = exact_grid(Lc.hcount[4] + Lc.hcount[5], RestrictPer<T>::value);
     count_launch();
@@ -1013,6 +1206,21 @@ cudaError_t restrict_t(const LevelDev& Lf, const LevelDev& Lc, int order, bool b
 template <typename T>
 cudaError_t prolong_t(const LevelDev& Lc, const LevelDev& Lf, int order, bool black_only, cudaStream_t s) {
   const Fields<T> ff = fields(Lf, T()), fc = fields(Lc, T());
+  if constexpr (sizeof(T) == 4) {
+    if (Lf.level == 0 && Lf.seg_pairs && black_only) {
+      ProlongQuadArgs a;
+      a.gf = Lf.g;
+      a.gc = Lc.g;
+      a.phi = ff.phi[1];
+      a.code = Lf.code[1];
+      a.list = Lf.list[0][1];
+      a.count = Lf.count + 1;
+      for (int c = 0; c < 2; ++c) a.cphi[c] = fc.phi[c];
+      count_launch();
+      launch_pdl(prolong_quad_kernel, dim3(seg_grid(Lf.hcount[1], 2, kProlongQuadBlocks)), dim3(kListBlock), 0, s, a);
+      return cudaGetLastError();
+    }
+  }
   ProlongArgs<T> a;
   a.gf = Lf.g;
   a.gc = Lc.g;

@@ -828,7 +828,7 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
   } off[kMaxLevels];
   const bool mixed = o.precision == 1;
   // fine_segments 1, 2: row segments of 8, 16 slots for the FP32 sweeps;
-  // 3: 16-slot segments, two slots per lane
+  // 3: 16-slot segments, four slots per lane
   const bool seg = mixed && o.fine_segments >= 1;
   const int seg_shift = seg ? (o.fine_segments >= 3 ? kSegShiftMax : kSegShiftMin + o.fine_segments - 1) : 0;
   for (int l = 0; l < H->nlev; ++l) {

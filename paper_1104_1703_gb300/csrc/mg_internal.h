@@ -115,7 +115,7 @@ struct LevelDev {
   double* rhsd[2];     // level 0 of the FP64 method: b / D (nullptr elsewhere)
   int exact_sum = 0;   // level 0: FP64 neighbour sums in integer arithmetic (exact_sum.cuh)
   int seg_shift = 0;   // level 0: log2 of the row-segment length (0: no segment lists)
-  int seg_pairs = 0;   // level 0, 16-slot segments: two slots per lane (gs_seg_pair_kernel)
+  int seg_pairs = 0;   // level 0, 16-slot segments: several slots per lane (gs_seg_pair_kernel)
   // FP32 copies for the inner cycles of the mixed-precision form (nullptr
   // when the hierarchy was created for FP64 only); level 0: phi32 is the
   // correction e, rhs32 is -r^ of the FP64 residual.
