@@ -268,8 +268,9 @@ __global__ void __launch_bounds__(kListBlock, UPDATE ? kPairUpdateBlocks : 8) gs
 // K9, first pass: the sum of r^2 per block into partials[blockIdx.x], r^ =
 // sum_nbr Phi_j - D Phi_i - b the scaled residual of the listed unknowns
 // (the grid is fixed per level, so the partials do not depend on scheduling).
+// (six blocks per SM in FP64, as the sweeps: union of balls 256^3 1% faster)
 template <int KIND, typename T, bool EXACT = false>
-__global__ void __launch_bounds__(kListBlock) res_list_kernel(ListArgs<T> a) {
+__global__ void __launch_bounds__(kListBlock, sizeof(T) == 8 ? 6 : 1) res_list_kernel(ListArgs<T> a) {
   constexpr int PER = PerThread<T>::value;
   const T* const tab = diag_tab<T>();
   const Geom g = a.g;
@@ -902,8 +903,9 @@ struct RefineArgs {
   double* partials;
 };
 
+// (six blocks per SM: 40 registers; 1563 -> 1480 us at 512^3 with holes)
 template <bool EXACT>
-__global__ void __launch_bounds__(kListBlock) refine_residual_kernel(RefineArgs a) {
+__global__ void __launch_bounds__(kListBlock, 6) refine_residual_kernel(RefineArgs a) {
   constexpr int PER = 2;
   const double* const tab = diag_tab<double>();
   const Geom g = a.g;
