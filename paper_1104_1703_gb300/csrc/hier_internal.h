@@ -39,6 +39,12 @@ struct mg_hierarchy {
   cudaStream_t cur = nullptr;          // stream the emitters launch on (stream, or cap_stream while capturing)
   cudaStream_t cap_stream = nullptr;
   GraphSlot graphs[3][2];              // [order][timing]
+  // a solve's cycles as one graph, per order: the pinned state, its device
+  // copy and whether the driver took the graph
+  GraphSlot loops[3];
+  gbmg::CycleLoop* hloop = nullptr;
+  gbmg::CycleLoop* dloop = nullptr;
+  bool loop_ok = true;
   std::vector<TimedPair>* cap_events = nullptr;
   size_t cap_events_used = 0;
   bool own_stream = false;

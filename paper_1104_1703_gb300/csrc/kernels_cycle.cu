@@ -870,8 +870,10 @@ __global__ void __launch_bounds__(kNormThreads) rhsnorm_kernel(NormArgs a) {
 // independent accumulators per thread so that the loads overlap).
 constexpr int kFinalThreads = 1024;
 
+// With LOOP thread 0 then decides whether the graph's loop runs another cycle.
+template <bool LOOP>
 __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const double* __restrict__ partials, int n,
-                                                                 double* out) {
+                                                                 double* out, LoopEnd loop) {
   pdl_wait();
   double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
   int e = threadIdx.x;
@@ -883,6 +885,24 @@ __global__ void __launch_bounds__(kFinalThreads) finalize_kernel(const double* _
   }
   for (; e < n; e += kFinalThreads) a0 += partials[e];
   block_reduce_store((a0 + a1) + (a2 + a3), out);
+  if (LOOP && threadIdx.x == 0) {
+    CycleLoop& st = *loop.state;
+    const double r = sqrt(*out) / st.h2;
+    const int done = st.n;
+    bool more = isfinite(r) && !(r / st.r_zero < st.tol);
+    if (st.may_switch && r >= st.floor && r / st.r_prev > st.eta_step) more = false;
+    st.r[done] = r;
+    st.r_prev = r;
+    st.n = done + 1;
+    cudaGraphSetConditional(loop.handle, more && done + 1 < st.budget ? 1u : 0u);
+  }
+}
+
+// the end of a norm: partial sums to *out, and the loop's decision
+void launch_finalize(const double* partials, int n, double* out, LoopEnd loop, cudaStream_t s) {
+  count_launch();
+  if (loop.state) launch_pdl(finalize_kernel<true>, dim3(1), dim3(kFinalThreads), 0, s, partials, n, out, loop);
+  else launch_pdl(finalize_kernel<false>, dim3(1), dim3(kFinalThreads), 0, s, partials, n, out, loop);
 }
 
 // Mixed precision, start of a refinement step: the FP64 scaled residual of
@@ -1785,7 +1805,7 @@ int residual_norm_blocks(const Geom& g) {
 }
 
 cudaError_t launch_residual_norm2(const LevelDev& L0, bool red_only, bool with_phi, double* partials,
-                                  int max_partials, double* out, cudaStream_t s) {
+                                  int max_partials, double* out, cudaStream_t s, LoopEnd loop) {
   int blocks;
   if (!with_phi) {
     NormArgs a;
@@ -1811,13 +1831,12 @@ cudaError_t launch_residual_norm2(const LevelDev& L0, bool red_only, bool with_p
       else launch_pdl(res_list_kernel<0, double>, dim3(grid), dim3(kListBlock), 0, s, a);
     }
   }
-  count_launch();
-  launch_pdl(finalize_kernel, dim3(1), dim3(kFinalThreads), 0, s, partials, blocks, out);
+  launch_finalize(partials, blocks, out, loop, s);
   return cudaGetLastError();
 }
 
 cudaError_t launch_refine_residual(const LevelDev& L0, double* partials, int max_partials, double* out,
-                                   cudaStream_t s) {
+                                   cudaStream_t s, LoopEnd loop) {
   RefineArgs a;
   a.g = L0.g;
   for (int c = 0; c < 2; ++c) {
@@ -1832,10 +1851,9 @@ cudaError_t launch_refine_residual(const LevelDev& L0, double* partials, int max
   a.partials = partials;
   const int blocks = 2 * list_grid(L0.g);
   if (blocks > max_partials) return cudaErrorInvalidValue;
-  count_launch(2);
+  count_launch();
   if (L0.exact_sum) launch_pdl(refine_residual_kernel<true>, dim3(blocks), dim3(kListBlock), 0, s, a);
-  else launch_pdl(refine_residual_kernel<false>, dim3(blocks), dim3(kListBlock), 0, s, a);
-  launch_pdl(finalize_kernel, dim3(1), dim3(kFinalThreads), 0, s, partials, blocks, out);
+  else launch_pdl(refine_residual_kernel<false>, dim3(blocks), dim3(kListBlock), 0, s, a);  launch_finalize(partials, blocks, out, loop, s);
   return cudaGetLastError();
 }
 

@@ -254,8 +254,32 @@ cudaError_t launch_prolong(const LevelDev& Lc, const LevelDev& Lf, int order, in
 // Sum of squares of the scaled residual of level 0 into partials[0..nblocks),
 // then a fixed-order reduction into out[0].  red_only as black_zero above.
 // with_phi = false evaluates the residual of Phi = 0 (i.e. of the rhs alone).
+// State of a solve's cycles run as one graph (a conditional while node): the
+// host writes it, the finalize kernel of every cycle adds the cycle's residual
+// norm and decides, by the host's rule and in its arithmetic, whether another
+// cycle follows.
+constexpr int kLoopMax = 64;  // cycles per launch
+struct CycleLoop {
+  double h2;        // h * h
+  double r_zero;    // ||r(Phi = 0)||
+  double tol;
+  double floor;     // no order switch below this norm
+  double eta_step;  // ratio of successive norms above which the order is switched
+  double r_prev;
+  int may_switch;
+  int budget;       // cycles at most, <= kLoopMax
+  int n;            // cycles done
+  int pad;
+  double r[kLoopMax];  // their residual norms
+};
+// where a cycle's norm goes on: nowhere (a single cycle) or into the loop
+struct LoopEnd {
+  CycleLoop* state = nullptr;
+  cudaGraphConditionalHandle handle = 0;
+};
+
 cudaError_t launch_residual_norm2(const LevelDev& L0, bool red_only, bool with_phi, double* partials,
-                                  int max_partials, double* out, cudaStream_t s);
+                                  int max_partials, double* out, cudaStream_t s, LoopEnd loop = LoopEnd());
 // One multigrid iteration with n_cycles coarse iterations per level (1: V,
 // 2 or more: W) on levels lb .. deepest in one CTA, for small levels (every
 // level lb..deepest satisfies small_level); lb >= 1.
@@ -283,7 +307,7 @@ cudaError_t launch_mid(const LevelDev* levels, int m, int lb, int deepest, int o
 // right-hand side -r^ and zero FP32 correction, plus the norm (like
 // launch_residual_norm2); and Phi += e in FP64.
 cudaError_t launch_refine_residual(const LevelDev& L0, double* partials, int max_partials, double* out,
-                                   cudaStream_t s);
+                                   cudaStream_t s, LoopEnd loop = LoopEnd());
 cudaError_t launch_refine_update(const LevelDev& L0, cudaStream_t s);
 // rhsd = b / D over level 0 (no-op when the level has no rhsd).
 cudaError_t launch_scale_rhs(const LevelDev& L0, cudaStream_t s);
