@@ -224,18 +224,37 @@ __device__ __forceinline__ T p2_sum(const Geom& gc, const T* c0, const T* c1, in
 
 constexpr int kNormThreads = 256;
 
+// Sum of a block's values to *out.  Blocks of up to kReduceThreads threads (the
+// norms' many blocks) add through shared memory in warp 0, one addition per
+// eight warps' values and five across its lanes: 12 FP64 warp instructions for
+// 256 threads, 45 with every warp reducing its own (each holds the FP64 pipe as
+// long as a whole warp of residuals).  The one large block of the final
+// sum keeps the shuffles, whose chain of dependent additions is shorter.
+constexpr int kReduceThreads = 512;
+
 __device__ __forceinline__ void block_reduce_store(double acc, double* out) {
-  __shared__ double warp_sums[32];
+  __shared__ double values[kReduceThreads];
   const int t = threadIdx.x + threadIdx.y * blockDim.x;
-  const int nw = (blockDim.x * blockDim.y) >> 5;
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-  if ((t & 31) == 0) warp_sums[t >> 5] = acc;
-  __syncthreads();
-  if (t < 32) {
-    double v = t < nw ? warp_sums[t] : 0.0;
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    if (t == 0) *out = v;
+  const int n = blockDim.x * blockDim.y;
+  if (n > kReduceThreads) {
+    for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+    if ((t & 31) == 0) values[t >> 5] = acc;
+    __syncthreads();
+    if (t >= 32) return;
+    acc = t < (n >> 5) ? values[t] : 0.0;
+  } else {
+    values[t] = acc;
+    __syncthreads();
+    if (t >= 32) return;
+    double a0 = acc, a1 = 0.0;
+    for (int i = t + 32; i < n; i += 64) {
+      a1 += values[i];
+      if (i + 32 < n) a0 += values[i + 32];
+    }
+    acc = a0 + a1;
   }
+  for (int off = 16; off > 0; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
+  if (t == 0) *out = acc;
 }
 
 // ---------------------------------------------------------------------------
