@@ -670,8 +670,13 @@ struct ProlongArgs {
 // black neighbours without reading the red value, so correcting the red
 // unknowns first would not change the result.
 template <typename T>
-__global__ void __launch_bounds__(kListBlock) prolong_list_kernel(ProlongArgs<T> a) {
-  constexpr int PER = 2;
+struct ProlongPer {  // fine unknowns per thread: FP64 hides its latency with more warps instead
+  static constexpr int value = sizeof(T) == 8 ? 1 : 2;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(kListBlock, sizeof(T) == 8 ? 8 : 1) prolong_list_kernel(ProlongArgs<T> a) {
+  constexpr int PER = ProlongPer<T>::value;
   const Geom gf = a.gf;
   const uint32_t n0 = a.skip_red ? 0u : *a.count[0], n = n0 + *a.count[1];
   const uint32_t stride = gridDim.x * kListBlock;
@@ -1256,7 +1261,7 @@ cudaError_t prolong_t(const LevelDev& Lc, const LevelDev& Lf, int order, bool bl
   a.skip_red = black_only ? 1 : 0;
   const uint32_t n = (black_only ? 0u : Lf.hcount[lo * 2]) + Lf.hcount[lo * 2 + 1];
   count_launch();
-  launch_pdl(prolong_list_kernel<T>, dim3(exact_grid(n, 2)), dim3(kListBlock), 0, s, a);
+  launch_pdl(prolong_list_kernel<T>, dim3(exact_grid(n, ProlongPer<T>::value)), dim3(kListBlock), 0, s, a);
   return cudaGetLastError();
 }
 
