@@ -72,13 +72,13 @@ cudaError_t launch_batch_gs(const Chunk* chunks, int nchunks, const PatchLevel* 
 // Level-0 chunks: mode 1: per-chunk sum of r^2 into partials[chunk]; 2:
 // per-chunk sum of b^2 (the residual of Phi = 0).
 cudaError_t launch_batch_norm(const Chunk* chunks, int nchunks, const PatchLevel* pls, const int* state, int mode,
-                              double* partials, int threads, int grid, cudaStream_t s);
+                              bool exact, double* partials, int threads, int grid, cudaStream_t s);
 // Residual and R1 into the coarse level of each chunk (coarse-list chunks).
 // Level-0 chunks: rhsd = b / D of their unknowns (every patch).
 cudaError_t launch_batch_scale(const Chunk* chunks, int nchunks, const PatchLevel* pls, int threads, int grid,
                                cudaStream_t s);
 cudaError_t launch_batch_restrict(const Chunk* chunks, int nchunks, const PatchLevel* pls, const int* state,
-                                  bool black_zero, int threads, int grid, cudaStream_t s);
+                                  bool black_zero, bool exact, int threads, int grid, cudaStream_t s);
 cudaError_t launch_batch_prolong(const Chunk* chunks, int nchunks, const PatchLevel* pls, const int* state,
                                  int threads, int grid, cudaStream_t s);
 // One CTA per patch: its bottom V-cycle in its current order.

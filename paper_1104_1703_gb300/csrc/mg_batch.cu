@@ -345,7 +345,8 @@ mg_status emit_smooth(mg_batch* B, int l, int sweeps, cudaStream_t s) {
 // (mode 1: residual, 2: right-hand side), then its copy to h_norm2.
 mg_status emit_norm(mg_batch* B, int mode, cudaStream_t s) {
   const Table& T = B->norm0;
-  BCKS(lok(B, launch_batch_norm(B->d_chunks + T.off, T.n, B->d_pls, B->d_state, mode, B->d_partials,
+  BCKS(lok(B, launch_batch_norm(B->d_chunks + T.off, T.n, B->d_pls, B->d_state, mode,
+                                B->opt.fp64_sum == 1, B->d_partials,
                                 B->tune.threads, grid_of(B, T), s),
            "batched norm"));
   BCKS(lok(B, launch_batch_patch_sums(B->d_partials, B->d_first, B->d_count, B->n, B->d_norm2, s), "patch sums"));
@@ -363,7 +364,8 @@ mg_status emit_cycle(mg_batch* B, cudaStream_t s) {
   for (int l = 0; l < B->lmax; ++l) {
     BCKS(emit_smooth(B, l, t.n_pre, s));  // step 1
     const Table& R = B->restr[l];
-    BCKS(lok(B, launch_batch_restrict(B->d_chunks + R.off, R.n, B->d_pls, B->d_state, black_zero, t.threads,
+    BCKS(lok(B, launch_batch_restrict(B->d_chunks + R.off, R.n, B->d_pls, B->d_state, black_zero,
+                                    l == 0 && B->opt.fp64_sum == 1, t.threads,
                                       grid_of(B, R), s),
              "batched residual and restriction"));  // steps 2-5
   }
