@@ -721,6 +721,37 @@ __global__ void __launch_bounds__(kListBlock, sizeof(T) == 8 ? 8 : 1) prolong_li
   }
 }
 
+// K6 on a large FP64 level 0: the same, two successive list entries per thread
+// (p2_pair).  Solve of 161x200x143 with holes: 15.04 -> 14.80 ms.
+__global__ void __launch_bounds__(kListBlock, 5) prolong_list_pairs_kernel(ProlongArgs<double> a) {
+  const uint32_t n0 = a.skip_red ? 0u : *a.count[0], n1 = *a.count[1];
+  const uint32_t h0 = (n0 + 1) / 2, h = h0 + (n1 + 1) / 2;
+  const uint32_t stride = gridDim.x * kListBlock;
+  uint32_t i = blockIdx.x * kListBlock + threadIdx.x;
+  // the entries are constant during a solve: the first round's are loaded
+  // before the wait on the previous kernel
+  uint32_t e0 = 0u, e1 = 0u;
+  auto entries = [&](uint32_t t) {
+    if (t >= h) return;
+    const int c = t >= h0;
+    const uint32_t at = 2 * (c ? t - h0 : t), n = c ? n1 : n0;
+    e0 = a.list[c][at];
+    e1 = at + 1 < n ? a.list[c][at + 1] : e0;
+  };
+  entries(i);
+  pdl_wait();
+  for (; i < h; i += stride, entries(i)) {
+    if (!entry_ok(a.gf, e0 & kListAt, 6) || !entry_ok(a.gf, e1 & kListAt, 6)) continue;
+    double* const phi = a.phi[i >= h0];
+    const uint32_t s0 = e0 & kListAt, s1 = e1 & kListAt;
+    const double old0 = phi[s0], old1 = phi[s1];
+    double w0, w1;
+    p2_pair(a.gf, a.gc, a.cphi[0], a.cphi[1], e0, e1, w0, w1);
+    phi[s0] = fma(w0, 1.0 / 64.0, old0);
+    if (e1 != e0) phi[s1] = fma(w1, 1.0 / 64.0, old1);
+  }
+}
+
 // K6 on the black unknowns of level 0 in the mixed form's FP32 cycles, over
 // the 16-slot row segments of the sweeps (gs_seg_pair_kernel): a lane takes
 // four consecutive slots of a row.  Their stencils share the four coarse rows
@@ -1261,6 +1292,14 @@ cudaError_t prolong_t(const LevelDev& Lc, const LevelDev& Lf, int order, bool bl
   a.skip_red = black_only ? 1 : 0;
   const uint32_t n = (black_only ? 0u : Lf.hcount[lo * 2]) + Lf.hcount[lo * 2 + 1];
   count_launch();
+  if constexpr (sizeof(T) == 8) {
+    // two unknowns per thread where that leaves every SM its threads (at 240
+    // thousand unknowns W-cycles are 0.5% slower with it)
+    if (Lf.level == 0 && n >= 8u * (uint32_t)device_sms() * kListBlock) {
+      launch_pdl(prolong_list_pairs_kernel, dim3(exact_grid((n + 3) / 2, 1)), dim3(kListBlock), 0, s, a);
+      return cudaGetLastError();
+    }
+  }
   launch_pdl(prolong_list_kernel<T>, dim3(exact_grid(n, ProlongPer<T>::value)), dim3(kListBlock), 0, s, a);
   return cudaGetLastError();
 }
