@@ -268,9 +268,9 @@ __global__ void __launch_bounds__(kListBlock, UPDATE ? kPairUpdateBlocks : 8) gs
 // K9, first pass: the sum of r^2 per block into partials[blockIdx.x], r^ =
 // sum_nbr Phi_j - D Phi_i - b the scaled residual of the listed unknowns
 // (the grid is fixed per level, so the partials do not depend on scheduling).
-// (six blocks per SM in FP64, as the sweeps: union of balls 256^3 1% faster)
+// (in FP64 eight blocks per SM: solves of 256^3 1.3% faster than with four)
 template <int KIND, typename T, bool EXACT = false>
-__global__ void __launch_bounds__(kListBlock, sizeof(T) == 8 ? 6 : 1) res_list_kernel(ListArgs<T> a) {
+__global__ void __launch_bounds__(kListBlock, sizeof(T) == 8 ? 8 : 1) res_list_kernel(ListArgs<T> a) {
   constexpr int PER = PerThread<T>::value;
   const T* const tab = diag_tab<T>();
   const Geom g = a.g;
@@ -959,9 +959,9 @@ struct RefineArgs {
   double* partials;
 };
 
-// (six blocks per SM: 40 registers; 1563 -> 1480 us at 512^3 with holes)
+// (eight blocks per SM: the mixed solve of 512^3 with holes 109.2 -> 108.0 ms)
 template <bool EXACT>
-__global__ void __launch_bounds__(kListBlock, 6) refine_residual_kernel(RefineArgs a) {
+__global__ void __launch_bounds__(kListBlock, 8) refine_residual_kernel(RefineArgs a) {
   constexpr int PER = 2;
   const double* const tab = diag_tab<double>();
   const Geom g = a.g;

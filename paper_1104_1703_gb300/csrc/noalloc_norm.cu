@@ -60,9 +60,13 @@ __device__ __forceinline__ double twice(double x) {
 // warp takes kTile cells of a row, lists the active ones and works with every
 // lane in use, and the six terms are added in integer arithmetic
 // (exact_sum.cuh), which leaves three FP64 instructions per active cell.
-constexpr int kTile = 128;
+// What is left are chains of dependent loads (mask, list, neighbours' masks,
+// values): eight blocks per SM at 32 registers and tiles of 256 cells hide
+// them (172 us; with four blocks of 64 registers and 128 cells 247).
+constexpr int kTile = 256;
+constexpr int kBlocksPerSm = 8;
 
-__global__ void __launch_bounds__(kNoAllocThreads)
+__global__ void __launch_bounds__(kNoAllocThreads, kBlocksPerSm)
 noalloc_resnorm_kernel(const int8_t* __restrict__ mask, const double* __restrict__ phi,
                        const double* __restrict__ rho, const double* __restrict__ bx,
                        const double* __restrict__ by, const double* __restrict__ bz, int nx, int ny, int nz,
@@ -182,10 +186,10 @@ extern "C" mg_status mg_residual_norm_noalloc(const int8_t* mask, const double* 
     set_thread_error("mg_residual_norm_noalloc: cudaGetSymbolAddress of the scratch array failed");
     return MG_ERR_CUDA;
   }
-  // a warp per tile of a row, at most 8 resident blocks per multiprocessor
+  // a warp per tile of a row, at most the resident blocks
   const long long tiles = (long long)((nx + kTile - 1) / kTile) * ny * nz;
   long long blocks = (tiles + kNoAllocThreads / 32 - 1) / (kNoAllocThreads / 32);
-  if (blocks > 8LL * device_sms()) blocks = 8LL * device_sms();
+  if (blocks > (long long)kBlocksPerSm * device_sms()) blocks = (long long)kBlocksPerSm * device_sms();
   if (blocks > kNoAllocMaxPartials) blocks = kNoAllocMaxPartials;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const double h2 = h * h;
