@@ -57,10 +57,11 @@ size_t batch_bottom_args_bytes();
 // patch whose deepest level is level 0 (the CTA then sweeps level 0
 // coarse_sweeps times).  Returns the dynamic shared memory the slot needs
 // (0 if it runs from global memory), or kBottomTooDeep when lb..deepest
-// holds more levels than the bottom cycle takes.
+// holds more levels than the bottom cycle takes.  cmat, cmat_n: the coarsest
+// solve's precomputed map and its unknowns per colour, or nullptr.
 constexpr size_t kBottomTooDeep = ~(size_t)0;
 size_t batch_fill_bottom(void* host_args, int slot, const LevelDev* levels, int lb, int deepest, int order,
-                         int n_pre, int n_post, int coarse_sweeps, int patch);
+                         int n_pre, int n_post, int coarse_sweeps, const double* cmat, const uint32_t* cmat_n);
 
 cudaError_t init_batch_kernels();
 int batch_grid(int nchunks, int threads, int persistent_ctas);

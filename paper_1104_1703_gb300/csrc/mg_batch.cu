@@ -282,8 +282,12 @@ mg_status build_tables(mg_batch* B) {
     for (int o = 1; o <= 2; ++o) {
       const int d = B->deepest[o - 1][p];
       const int lb = d == 0 ? 0 : B->lb[o - 1][p];
+      // the patch's own map of its coarsest solve, when it is of these sweeps
+      const bool map = H->cmat_ok[o] && H->cmat_prec == kFP64 && d == H->deepest[o] &&
+                       H->opt.coarse_sweeps == B->opt.coarse_sweeps;
       const size_t sm = batch_fill_bottom(bot.data(), 2 * p + o - 1, H->L, lb, d, o, t.n_pre, t.n_post,
-                                          B->opt.coarse_sweeps, p);
+                                          B->opt.coarse_sweeps, map ? (const double*)H->cmat[o] : nullptr,
+                                          H->cmat_n[o]);
       if (sm == kBottomTooDeep)
         return bfail(B, MG_ERR_INVALID_ARG, "patch " + std::to_string(p) + ": too many levels below bottom_slots");
       B->bottom_smem = std::max(B->bottom_smem, sm);
