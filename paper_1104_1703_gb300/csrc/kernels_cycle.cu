@@ -456,8 +456,11 @@ __device__ __forceinline__ T child_residual_sum(const RestrictArgs<T>& a, const 
 // the last fine operation was a complete red-black sweep, after which every
 // black cell satisfies its own equation: only red children carry a
 // residual.  Children outside the active set (of this order) count 0.
+// Bound by load latency: a full SM of threads in FP32, half of one in FP64
+// (more would spill) instead of what 40 to 100 registers leave: mixed solves of
+// 256^3 0.4%, FP64 W-cycles at 128^3 0.5% faster.
 template <int KIND, bool BLACK_ZERO, typename T>
-__global__ void __launch_bounds__(kBlockX * kBlockY) restrict_kernel(RestrictArgs<T> a) {
+__global__ void __launch_bounds__(kBlockX * kBlockY, sizeof(T) == 4 ? 16 : 8) restrict_kernel(RestrictArgs<T> a) {
   const T* const tab = diag_tab<T>();
   const Geom gc = a.gc;
   const int I = blockIdx.x * kBlockX + threadIdx.x;
