@@ -268,48 +268,33 @@ __global__ void __launch_bounds__(kListBlock, UPDATE ? kPairUpdateBlocks : 8) gs
 // K9, first pass: the sum of r^2 per block into partials[blockIdx.x], r^ =
 // sum_nbr Phi_j - D Phi_i - b the scaled residual of the listed unknowns
 // (the grid is fixed per level, so the partials do not depend on scheduling).
-// (in FP64 eight blocks per SM: solves of 256^3 1.3% faster than with four)
+// One unknown per thread and eight blocks per SM: with two and 64 registers
+// FP64 solves of 256^3 were 2.5% slower.
 template <int KIND, typename T, bool EXACT = false>
 __global__ void __launch_bounds__(kListBlock, sizeof(T) == 8 ? 8 : 1) res_list_kernel(ListArgs<T> a) {
-  constexpr int PER = PerThread<T>::value;
   const T* const tab = diag_tab<T>();
-  const Geom g = a.g;
+  const Geom& g = a.g;
   const uint32_t n = *a.count;
   const uint32_t stride = gridDim.x * kListBlock;
-  uint32_t base = blockIdx.x * kListBlock + threadIdx.x;
-  // list entries and diagonals are fixed by the mask: loaded before the wait
-  // on the previous kernel (first round) and during the current round (next)
-  uint32_t e[PER];
-  T d[PER];
-  auto invariants = [&](uint32_t b0) {
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      const uint32_t i = b0 + u * stride;
-      e[u] = i < n ? a.list[i] : 0u;
-      d[u] = i < n ? diag_of<KIND>(KIND == 0 ? a.code[e[u] & kListAt] : 0, a.diag, e[u] & kListAt, tab) : T(0);
-    }
+  // the list entry and the diagonal are fixed by the mask: loaded before the
+  // wait on the previous kernel (first round) and during the current one (next)
+  uint32_t i = blockIdx.x * kListBlock + threadIdx.x, next = 0u;
+  T dnext = T(0);
+  auto invariants = [&](uint32_t k) {
+    next = k < n ? a.list[k] : 0u;
+    dnext = k < n ? diag_of<KIND>(KIND == 0 ? a.code[next & kListAt] : 0, a.diag, next & kListAt, tab) : T(0);
   };
-  invariants(base);
+  invariants(i);
   pdl_wait();
   double acc = 0.0;
-  for (; base < n; base += PER * stride) {
-    long long at[PER];
-    T r[PER];
-    bool ok[PER];
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      ok[u] = base + u * stride < n;
-      at[u] = e[u] & kListAt;
-      ok[u] = ok[u] && entry_ok(g, at[u], 4);
-      if (ok[u]) {
-        const T s = nbr_sum_sel<EXACT>(a.other, at[u], (e[u] & kListPlusX) ? 1 : -1, g.P, g.sz);
-        r[u] = fma(-d[u], a.self[at[u]], s) - a.rhs[at[u]];
-      }
-    }
-    invariants(base + PER * stride);
-#pragma unroll
-    for (int u = 0; u < PER; ++u)
-      if (ok[u]) acc = fma((double)r[u], (double)r[u], acc);
+  for (; i < n; i += stride) {
+    const uint32_t e = next, at = e & kListAt;
+    const T d = dnext;
+    invariants(i + stride);
+    if (!entry_ok(g, at, 4)) continue;
+    const T s = nbr_sum_sel32<EXACT>(a.other, at, x_nbr(e, at), (uint32_t)g.P, (uint32_t)g.sz);
+    const T r = fma(-d, a.self[at], s) - a.rhs[at];
+    acc = fma((double)r, (double)r, acc);
   }
   block_reduce_store(acc, a.partials + blockIdx.x);
 }
@@ -938,58 +923,32 @@ struct RefineArgs {
   double* partials;
 };
 
-// (eight blocks per SM: the mixed solve of 512^3 with holes 109.2 -> 108.0 ms)
+// One unknown per thread and eight blocks per SM: with two and 64 registers the
+// mixed solve of 512^3 with holes took 109.2 ms, now 106.5.
 template <bool EXACT>
 __global__ void __launch_bounds__(kListBlock, 8) refine_residual_kernel(RefineArgs a) {
-  constexpr int PER = 2;
   const double* const tab = diag_tab<double>();
-  const Geom g = a.g;
+  const Geom& g = a.g;
   const uint32_t n0 = *a.count[0], n = n0 + *a.count[1];
   const uint32_t stride = gridDim.x * kListBlock;
-  uint32_t base = blockIdx.x * kListBlock + threadIdx.x;
-  // list entries and diagonals are fixed by the mask: the first round's are
-  // loaded before the wait on the previous kernel; each next round's
-  // entries while the current one computes, its diagonals with its data
-  uint32_t e[PER];
-  double D[PER];
-  auto entry = [&](uint32_t i) { return i < n ? (i >= n0 ? a.list[1][i - n0] : a.list[0][i]) : 0u; };
-#pragma unroll
-  for (int u = 0; u < PER; ++u) e[u] = entry(base + u * stride);
-#pragma unroll
-  for (int u = 0; u < PER; ++u) {
-    const uint32_t i = base + u * stride;
-    D[u] = i < n ? tab[8 + __popc((unsigned)a.code[i >= n0][e[u] & kListAt] >> kGhostShift)] : 0.0;
-  }
+  uint32_t i = blockIdx.x * kListBlock + threadIdx.x;
+  // list entries are fixed by the mask: the first is loaded before the wait
+  // on the previous kernel, each next one while the current one computes
+  auto entry = [&](uint32_t k) { return k < n ? (k >= n0 ? a.list[1][k - n0] : a.list[0][k]) : 0u; };
+  uint32_t next = entry(i);
   pdl_wait();
   double acc = 0.0;
-  for (bool first = true; base < n; base += PER * stride, first = false) {
-    long long at[PER];
-    int cc[PER];
-    double r[PER];
-    bool ok[PER];
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      const uint32_t i = base + u * stride;
-      ok[u] = i < n;
-      if (!ok[u]) continue;
-      const int c = i >= n0;
-      cc[u] = c;
-      at[u] = e[u] & kListAt;
-      ok[u] = entry_ok(g, at[u], 7);
-      if (!ok[u]) continue;
-      const double s = nbr_sum_sel<EXACT>(a.phi[1 - c], at[u], (e[u] & kListPlusX) ? 1 : -1, g.P, g.sz);
-      const double Du = first ? D[u] : tab[8 + __popc((unsigned)a.code[c][at[u]] >> kGhostShift)];
-      r[u] = fma(-Du, a.phi[c][at[u]], s) - a.rhs[c][at[u]];
-    }
-#pragma unroll
-    for (int u = 0; u < PER; ++u) e[u] = entry(base + PER * stride + u * stride);
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-      if (!ok[u]) continue;
-      a.rhs32[cc[u]][at[u]] = narrow_f64(-r[u]);
-      a.e32[cc[u]][at[u]] = 0.0f;
-      acc = fma(r[u], r[u], acc);
-    }
+  for (; i < n; i += stride) {
+    const uint32_t e = next, at = e & kListAt;
+    next = entry(i + stride);
+    if (!entry_ok(g, at, 7)) continue;
+    const int c = i >= n0;
+    const double s = nbr_sum_sel32<EXACT>(a.phi[1 - c], at, x_nbr(e, at), (uint32_t)g.P, (uint32_t)g.sz);
+    const double D = tab[8 + __popc((unsigned)a.code[c][at] >> kGhostShift)];
+    const double r = fma(-D, a.phi[c][at], s) - a.rhs[c][at];
+    a.rhs32[c][at] = narrow_f64(-r);
+    a.e32[c][at] = 0.0f;
+    acc = fma(r, r, acc);
   }
   block_reduce_store(acc, a.partials + blockIdx.x);
 }
@@ -1019,11 +978,12 @@ int kind_of(int level, int order) { return level == 0 ? 0 : (order == 1 ? 2 : 1)
 uint8_t bit_of(int level, int order) { return (level >= 1 && order == 1) ? kActive1 : kActive2; }
 
 // fixed grid of the norm kernels of a level: enough blocks for every slot of
-// one colour, at most 16 per SM (grid-stride beyond that)
+// one colour, at most the 8 per SM that are resident together (grid-stride
+// beyond that)
 int list_grid(const Geom& g) {
   const long long n = (long long)g.hx * g.ny * g.nz;
   long long b = (n + kListBlock - 1) / kListBlock;
-  const long long cap = 16LL * device_sms();
+  const long long cap = 8LL * device_sms();
   if (b > cap) b = cap;
   if (b < 1) b = 1;
   return (int)b;
