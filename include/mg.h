@@ -122,8 +122,8 @@ typedef enum { MG_MEM_HOST = 0, MG_MEM_DEVICE = 1 } mg_mem;
  *                  sweeps (built once per mask, one launch): a small
  *                  matrix-vector product instead of 2 * coarse_sweeps
  *                  dependent half-sweeps per visit, the same result up to
- *                  rounding; 0 = the sweeps.  (Batched patches use the
- *                  sweeps.) */
+ *                  rounding; 0 = the sweeps.  (Batched patches use their
+ *                  own maps.) */
 typedef struct {
   int n_pre, n_post, n_cycles, coarse_sweeps, hold_solves;
   double eta;
