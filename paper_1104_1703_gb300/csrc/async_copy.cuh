@@ -96,16 +96,22 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned b
 }
 
 // ---- tcgen05 (fifth-generation tensor cores, accumulators in TMEM) ----
+//
+// The .sync.aligned forms want the warp's lanes converged: a caller whose
+// lanes have just parted (one issuing lane, rows outside the grid) does not
+// have to join them itself, each of these waits for the whole warp first.
 
 // Allocates `ncols` TMEM columns (a power of two >= 32) for this CTA; the
 // whole warp executes it and the TMEM address lands in *dst (shared memory).
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(dst)), "r"(ncols)
                : "memory");
   asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
+  __syncwarp();
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
@@ -150,6 +156,7 @@ __device__ __forceinline__ void tc_commit(unsigned long long* bar) {
 // thread) into registers.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   uint32_t r[16];
+  __syncwarp();
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
       "%15}, [%16];"

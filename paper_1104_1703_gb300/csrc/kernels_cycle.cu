@@ -1283,6 +1283,7 @@ __device__ __forceinline__ T nbr_sum_cg(const T* o, long long at, int dx, int P,
 
 __device__ __forceinline__ void cluster_barrier() {
   __threadfence();
+  __syncwarp();  // the aligned forms want converged warps
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
