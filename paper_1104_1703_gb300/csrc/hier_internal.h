@@ -23,6 +23,7 @@ struct GraphSlot {
   cudaGraphExec_t exec = nullptr;
   int deepest = -2;                // deepest level at capture time
   unsigned long long lists_hash = 0;  // list lengths at capture time (they size the grids)
+  int n_pre = -1, n_post = -1;     // sweeps at capture time (a batch changes its patches')
   unsigned long long nodes = 0;    // kernel launches per replay
   std::vector<TimedPair> events;   // level-0 half-sweep event pairs (timing graphs)
 };

@@ -478,7 +478,9 @@ mg_status copy_phi(mg_batch* B, int p, bool to_save) {
   return MG_OK;
 }
 
-mg_status set_schedule(mg_batch* B, int n_pre, int n_post) {
+// The sweeps of the batch and of its patches' own cycles (whose captured
+// graphs carry the sweeps in their key).
+void set_schedule(mg_batch* B, int n_pre, int n_post) {
   B->tune.n_pre = n_pre;
   B->tune.n_post = n_post;
   B->opt.n_pre = n_pre;
@@ -486,14 +488,7 @@ mg_status set_schedule(mg_batch* B, int n_pre, int n_post) {
   for (mg_hierarchy* H : B->P) {
     H->opt.n_pre = n_pre;
     H->opt.n_post = n_post;
-    for (auto& row : H->graphs)
-      for (auto& gs : row) {
-        if (gs.exec) cudaGraphExecDestroy(gs.exec);
-        gs.exec = nullptr;
-        gs.deepest = -2;
-      }
   }
-  return MG_OK;
 }
 
 mg_status solve_impl(mg_batch* B, double tol, int max_cycles, mg_solve_info* infos) {
@@ -749,7 +744,7 @@ mg_status mg_batch_set_tuning(mg_batch* B, const mg_batch_tuning* t) {
   const double ms = t->ms_per_cycle;
   B->tune = *t;
   B->tune.ms_per_cycle = ms;
-  BCKS(set_schedule(B, t->n_pre, t->n_post));
+  set_schedule(B, t->n_pre, t->n_post);
   return build_tables(B);
 }
 

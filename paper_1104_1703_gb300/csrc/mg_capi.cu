@@ -430,6 +430,19 @@ void drop_graph(GraphSlot& g) {
   g.deepest = -2;
 }
 
+// What a captured cycle depends on besides the hierarchy's fixed options:
+// noted at its capture, and compared before it is replayed.
+void note_key(const mg_hierarchy* H, int order, GraphSlot& g) {
+  g.deepest = H->deepest[order];
+  g.lists_hash = H->lists_hash;
+  g.n_pre = H->opt.n_pre;
+  g.n_post = H->opt.n_post;
+}
+bool current(const mg_hierarchy* H, int order, const GraphSlot& g) {
+  return g.exec && g.deepest == H->deepest[order] && g.lists_hash == H->lists_hash && g.n_pre == H->opt.n_pre &&
+         g.n_post == H->opt.n_post;
+}
+
 // Enqueues the FP64 residual of the mixed form (which also writes the FP32
 // right-hand side -r^ and zeroes the FP32 correction) and its norm.
 mg_status emit_refine_residual(mg_hierarchy* H, LoopEnd loop = LoopEnd()) {
@@ -489,8 +502,7 @@ mg_status capture_cycle(mg_hierarchy* H, int order, GraphSlot& gs) {
   H->cap_events = nullptr;
   if (st != MG_OK) return st;
   if (e != cudaSuccess || !gs.exec) return cuda_fail(H, e, "graph capture");
-  gs.deepest = H->deepest[order];
-  gs.lists_hash = H->lists_hash;
+  note_key(H, order, gs);
   gs.nodes = t_captured;
   return MG_OK;
 }
@@ -557,8 +569,7 @@ bool capture_loop(mg_hierarchy* H, int order, GraphSlot& gs) {
     cudaGetLastError();
   }
   cudaGraphDestroy(graph);
-  gs.deepest = H->deepest[order];
-  gs.lists_hash = H->lists_hash;
+  note_key(H, order, gs);
   gs.nodes = t_captured;
   return gs.exec != nullptr;
 }
@@ -573,7 +584,7 @@ mg_status run_loop(mg_hierarchy* H, int order, int budget, bool* ran) {
   if (H->opt.precision == 1 && !H->prepared) CKS(emit_refine_residual(H));
   H->prepared = true;
   GraphSlot& gs = H->loops[order];
-  if (!gs.exec || gs.deepest != H->deepest[order] || gs.lists_hash != H->lists_hash)
+  if (!current(H, order, gs))
     H->loop_ok = capture_loop(H, order, gs);
   if (!H->loop_ok) return MG_OK;
   H->hloop->budget = std::min(budget, kLoopMax);
@@ -603,7 +614,7 @@ mg_status run_cycle(mg_hierarchy* H, int order, double* r_out) {
     CKS(emit_cycle(H, order));
   } else {
     GraphSlot& gs = H->graphs[order][H->timing ? 1 : 0];
-    if (!gs.exec || gs.deepest != H->deepest[order] || gs.lists_hash != H->lists_hash)
+    if (!current(H, order, gs))
       CKS(capture_cycle(H, order, gs));
     CK(H, cudaGraphLaunch(gs.exec, H->stream));
     count_launch(gs.nodes);
