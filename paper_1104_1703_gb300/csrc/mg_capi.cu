@@ -328,19 +328,28 @@ mg_status smooth(mg_hierarchy* H, int l, int order, int sweeps, int prec = kFP64
   return MG_OK;
 }
 
+// True when a cycle may run its coarse levels in a cluster: with sweeps on both
+// sides of the coarse correction (the cluster's red residuals take the place of
+// the red correction, and its messages of one kind need a step in between),
+// which a batch may take from its patches after their masks were built.
+bool cluster_runs(const mg_hierarchy* H) {
+  return H->cluster_ok && !H->opt.coarse_cluster && H->opt.n_pre >= 1 && H->opt.n_post >= 1;
+}
+
 // Section 2 recipe at level l, recursing N_cycles times into level l+1, in
 // FP64 or (inner cycles of the mixed form) FP32.
 mg_status iteration(mg_hierarchy* H, int l, int order, int prec = kFP64, bool update_last = false) {
   const mg_options& o = H->opt;
   // the coarsest solve's precomputed map, when it matches this solve
   const void* cmat = (H->cmat_ok[order] && H->cmat_prec == prec) ? H->cmat[order] : nullptr;
-  // the small coarse levels run as one single-CTA launch, which carries
-  // the N_cycles recursion below level l itself
-  if (l >= 1 && l == H->cl_plan[order].first && !o.coarse_cluster)
+  // the coarse levels that fit a cluster run as one launch of it, which
+  // carries the N_cycles recursion below level l itself
+  if (l >= 1 && l == H->cl_plan[order].first && cluster_runs(H))
     return launch_ok(H, launch_cluster_cycle(H->L, H->cl_plan[order], order, o.n_pre, o.n_post, o.coarse_sweeps,
                                              o.n_cycles, prec, H->cl_blobs[order], cmat, H->cmat_n[order],
                                              H->err_flag + 3, H->cur),
                      "coarse levels");
+  // without one, the small coarse levels run as one single-CTA launch
   if (l >= 1 && small_level(H->L[l].g))
     return launch_ok(H, launch_bottom(H->L, l, H->deepest[order], order, o.n_pre, o.n_post, o.coarse_sweeps,
                                       o.n_cycles, prec, cmat, H->cmat_n[order], H->cur),
@@ -707,12 +716,11 @@ mg_status build_levels(mg_hierarchy* H, bool fine_built = false, const int8_t* m
     H->deepest[o] = -1;
     for (int l = 0; l < H->nlev && H->active[o][l] > 0; ++l) H->deepest[o] = l;
   }
-  // the coarse levels that run as one cluster launch (its residuals take the
-  // place of the red correction, which needs sweeps on both sides)
+  // the coarse levels that run as one cluster launch
   const int prec = H->opt.precision == 1 ? kFP32 : kFP64;
   for (int o = 1; o <= 2; ++o) {
     H->cl_plan[o] = ClPlan();
-    if (!H->cluster_ok || H->opt.n_pre < 1 || H->opt.n_post < 1) continue;
+    if (!cluster_runs(H)) continue;
     H->cl_plan[o] = cluster_plan(H->L, H->deepest[o], o, prec, H->cl_bound);
     if (H->cl_plan[o].first)
       CKS(launch_ok(H, launch_cluster_build(H->L, H->cl_plan[o], o, prec, H->cl_blobs[o], s), "coarse-level records"));

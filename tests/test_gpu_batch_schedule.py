@@ -41,6 +41,13 @@ def test_patch_after_a_schedule_change(first, then):
     check_schedule_change(first, then)
 
 
+@pytest.mark.parametrize("first,then", [((2, 2), (0, 2)), ((2, 2), (2, 0)), ((1, 1), (0, 1)), ((0, 2), (2, 2)),
+                                        ((2, 0), (1, 1))])
+def test_one_sided_schedules_leave_the_cluster(first, then):
+    """Sweeps on one side only: the coarse levels run launch by launch, as in a hierarchy created so."""
+    check_schedule_change(first, then)
+
+
 def check_schedule_change(first, then):
     dev = torch.device("cuda:0")
     masks = [torch.from_numpy(w["mask"]).to(dev) for w in PATCHES]
