@@ -122,6 +122,7 @@ int conv_groups(const ConvArgs& a) {
 // at least three stages in shared memory.
 void conv_plan(ConvArgs& a) {
   constexpr size_t kBudget = 225 * 1024;  // dynamic shared memory
+  constexpr int kMaxCopySide = 256;       // of a TMA copy's box
   const unsigned wall = 27u * (unsigned)a.cin * (unsigned)a.cout * 2u;
   a.wres = wall <= 72u * 1024u ? 1 : 0;
   conv_chunks(a.cin, &a.span, &a.kc);
@@ -144,6 +145,7 @@ void conv_plan(ConvArgs& a) {
       a.bz = 1;
     } else {
       conv_tile_box(a.W, a.H, a.D, kConvTileM * a.group, &a.bx, &a.by, &a.bz);
+      if (a.group > 1 && (a.by > kMaxCopySide || a.bz > kMaxCopySide)) continue;  // a grid one or two voxels wide
     }
     stages();
     if (a.group == 1 || (a.stages >= (a.halo ? 2 : 3) && (a.halo || conv_groups(a) >= 100))) break;
