@@ -20,13 +20,18 @@
  *    or pinned host pointer) or device memory of the hierarchy's GPU
  *    (MG_MEM_DEVICE).  An MG_MEM_DEVICE pointer that is not device (or
  *    managed) memory of that GPU is refused with MG_ERR_INVALID_ARG before
- *    any copy or launch.  The caller owns every buffer it passes; the library
- *    copies what it needs before returning and never keeps a caller pointer.
- *    All library memory is device memory owned by the hierarchy.
+ *    any copy or launch.  The caller owns every buffer it passes and the
+ *    library never keeps a caller pointer.  Host buffers have been read or
+ *    written when the call returns; device buffers are read and written in
+ *    the order of the hierarchy's stream.  All library memory is device
+ *    memory owned by the hierarchy.
  *  - Work is issued on the hierarchy's CUDA stream.  Calls that return host
- *    data (solve, norms, copies to MG_MEM_HOST) synchronise that stream; calls
- *    that write device data into caller buffers (MG_MEM_DEVICE) are ordered
- *    on the stream and complete asynchronously.
+ *    data (solve, norms, copies to MG_MEM_HOST) and the two that take the
+ *    coarser level's potential (mg_set_dirichlet_from_coarse,
+ *    mg_faces_from_coarse) synchronise that stream, for any memory kind and
+ *    size; the other calls on caller buffers in device memory return before
+ *    the stream has reached them, so such a buffer is rewritten, freed or
+ *    read on another stream only after that stream waits for this one.
  *  - Values at inactive cells are ignored on input and written as 0 on output.
  *  - Every call returns an mg_status; nothing is thrown across the ABI.  On
  *    error mg_last_error() describes the failure.  A hierarchy stays usable
@@ -214,6 +219,7 @@ mg_status mg_set_dirichlet(mg_hierarchy* hier, const double* bx, const double* b
  *  ox, oy, oz   lower corner of coarse cell (0,0,0) in fine-cell units: the
  *               coarse cell (I,J,K) spans [ox+2I, ox+2I+2] x ... so its
  *               centre is at ox+2I+1.  Typical: -2 (one coarse ghost cell).
+ * phi_c has been read when the call returns.
  * Errors: INVALID_ARG (including a boundary face outside the coarse centres),
  * CUDA. */
 mg_status mg_set_dirichlet_from_coarse(mg_hierarchy* hier, const double* phi_c, mg_mem where, int cnx,
@@ -224,8 +230,9 @@ mg_status mg_set_dirichlet_from_coarse(mg_hierarchy* hier, const double* phi_c, 
  * domain gets the coarse potential trilinearly interpolated at its centre
  * (Section 1 one-way interface); every other face is 0.  bx, by, bz are
  * device buffers of the hierarchy's GPU ((nx+1) ny nz, nx (ny+1) nz,
- * nx ny (nz+1) doubles).  Errors: INVALID_ARG (including a boundary face
- * outside the coarse cell centres), CUDA. */
+ * nx ny (nz+1) doubles).  phi_c has been read and the faces are written when
+ * the call returns.  Errors: INVALID_ARG (including a boundary face outside
+ * the coarse cell centres), CUDA. */
 mg_status mg_faces_from_coarse(mg_hierarchy* hier, const double* phi_c, mg_mem where, int cnx, int cny, int cnz, int ox,
                                int oy, int oz, double* bx, double* by, double* bz);
 

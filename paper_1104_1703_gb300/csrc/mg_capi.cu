@@ -815,6 +815,16 @@ bool coarse_covers(const Geom& g, int cnx, int cny, int cnz, int ox, int oy, int
   return axis(g.nx, cnx, ox) && axis(g.ny, cny, oy) && axis(g.nz, cnz, oz);
 }
 
+// Waits until the coarse potential has been read: it belongs to another level,
+// whose program may write it on another stream once the call has returned.
+// *err: the flag of a face outside the coarse centres (covered: there is none).
+mg_status coarse_read(mg_hierarchy* H, bool covered, int* err) {
+  if (!covered) CK(H, cudaMemcpyAsync(H->hscal, H->err_flag, sizeof(int), cudaMemcpyDeviceToHost, H->stream));
+  CK(H, cudaStreamSynchronize(H->stream));
+  if (!covered) std::memcpy(err, H->hscal, sizeof(int));
+  return MG_OK;
+}
+
 mg_status check_level(mg_hierarchy* H, int level) {
   if (!H) return fail(H, MG_ERR_INVALID_ARG, "null hierarchy");
   if (level < 0 || level >= H->nlev) return fail(H, MG_ERR_INVALID_ARG, "level out of range");
@@ -1258,8 +1268,7 @@ mg_status mg_set_dirichlet_from_coarse(mg_hierarchy* H, const double* phi_c, mg_
   if (where == MG_MEM_HOST) CKS(ensure_staging(H, bytes));
   const void* src;
   CKS(device_view(H, phi_c, where, bytes, 0, &src));
-  // a coarse grid that covers every face of the box needs no look at the
-  // flag, so the call does not wait
+  // a coarse grid that covers every face of the box needs no look at the flag
   const bool covered = coarse_covers(H->L[0].g, cnx, cny, cnz, ox, oy, oz);
   if (!covered) CK(H, cudaMemsetAsync(H->err_flag, 0, sizeof(int), H->stream));
   H->bc_zero = false;
@@ -1269,14 +1278,8 @@ mg_status mg_set_dirichlet_from_coarse(mg_hierarchy* H, const double* phi_c, mg_
   CKS(launch_ok(H, launch_fold_coarse(H->L[0], H->F, (const double*)src, cnx, cny, cnz, ox, oy, oz, H->err_flag,
                                      H->stream),
                 "coarse interpolation"));
-  if (covered) {
-    if (where == MG_MEM_HOST) CK(H, cudaStreamSynchronize(H->stream));
-    return MG_OK;
-  }
   int err = 0;
-  CK(H, cudaMemcpyAsync(H->hscal, H->err_flag, sizeof(int), cudaMemcpyDeviceToHost, H->stream));
-  CK(H, cudaStreamSynchronize(H->stream));
-  std::memcpy(&err, H->hscal, sizeof(int));
+  CKS(coarse_read(H, covered, &err));
   if (err) {
     CKS(zero_split(H, H->L[0].g, H->F.bc));
     H->bc_zero = true;
@@ -1309,14 +1312,8 @@ mg_status mg_faces_from_coarse(mg_hierarchy* H, const double* phi_c, mg_mem wher
   CKS(launch_ok(H, launch_faces_from_coarse(H->L[0], (const double*)src, cnx, cny, cnz, ox, oy, oz, bx, by, bz,
                                             H->err_flag, H->stream),
                 "coarse interpolation"));
-  if (covered) {
-    if (where == MG_MEM_HOST) CK(H, cudaStreamSynchronize(H->stream));
-    return MG_OK;
-  }
   int err = 0;
-  CK(H, cudaMemcpyAsync(H->hscal, H->err_flag, sizeof(int), cudaMemcpyDeviceToHost, H->stream));
-  CK(H, cudaStreamSynchronize(H->stream));
-  std::memcpy(&err, H->hscal, sizeof(int));
+  CKS(coarse_read(H, covered, &err));
   if (err) return fail(H, MG_ERR_INVALID_ARG, "a boundary face lies outside the coarse cell centres");
   return MG_OK;
 }
