@@ -23,6 +23,7 @@
 #include "../../include/mg.h"
 #include "exact_sum.cuh"
 #include "mg_internal.h"
+#include "row_tiles.h"
 
 namespace gbmg {
 
@@ -57,19 +58,25 @@ __device__ __forceinline__ double twice(double x) {
 // A thread per cell ran about 12 FP64 operations for active and idle lanes
 // alike, on a pipe that takes 16 cycles per warp instruction (504 us on a
 // half-active 256^3 patch with face values, whose 688 MB take 102 us).  So a
-// warp takes kTile cells of a row, lists the active ones and works with every
-// lane in use, and the six terms are added in integer arithmetic
-// (exact_sum.cuh), which leaves three FP64 instructions per active cell.
+// warp takes kTile cells of a row, or of several short rows (row_tiles.h),
+// lists the active ones and works with every lane in use, and the six terms are
+// added in integer arithmetic (exact_sum.cuh), which leaves three FP64
+// instructions per active cell.
 // What is left are chains of dependent loads (mask, list, neighbours' masks,
 // values): eight blocks per SM at 32 registers and tiles of 256 cells hide
-// them (172 us; with four blocks of 64 registers and 128 cells 247).
+// them (172 us; with four blocks of 64 registers and 128 cells 247).  ROWS: a
+// tile has several rows, whose cells look up their own (half-active boxes, 512
+// x 512 rows of 8 cells: 38 us, a tile per row 176, a thread per cell 100; 256
+// x 256 rows of 48: 58, 56 and 153), as many as leave every resident warp a tile
+// (32 x 32 rows of 32: 16.5 us, with full tiles of eight rows 21.7).
 constexpr int kTile = 256;
 constexpr int kBlocksPerSm = 8;
 
+template <bool ROWS>
 __global__ void __launch_bounds__(kNoAllocThreads, kBlocksPerSm)
 noalloc_resnorm_kernel(const int8_t* __restrict__ mask, const double* __restrict__ phi,
                        const double* __restrict__ rho, const double* __restrict__ bx,
-                       const double* __restrict__ by, const double* __restrict__ bz, int nx, int ny, int nz,
+                       const double* __restrict__ by, const double* __restrict__ bz, RowTiles T, int ny, int nz,
                        double h2, double* partials) {
   constexpr int kWarps = kNoAllocThreads / 32;
   __shared__ uint8_t active[kWarps][kTile];
@@ -77,48 +84,54 @@ noalloc_resnorm_kernel(const int8_t* __restrict__ mask, const double* __restrict
   if (threadIdx.x < 8) diag[threadIdx.x] = (double)(6 + (int)threadIdx.x);
   __syncthreads();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int nx = (int)T.nx;
   const long long sy = nx, sz = (long long)nx * ny;
-  const unsigned tiles = (unsigned)(nx + kTile - 1) / kTile;
-  const unsigned n = tiles * (unsigned)ny * (unsigned)nz;
   double acc = 0.0;
-  for (unsigned t = blockIdx.x * kWarps + w; t < n; t += gridDim.x * kWarps) {
-    const unsigned row = t / tiles;
-    const int k = (int)(row / (unsigned)ny), j = (int)(row - (unsigned)k * (unsigned)ny);
-    const int i0 = (int)(t - row * tiles) * kTile;
-    const long long r0 = (long long)row * nx;  // cell (0, j, k)
-    const int8_t* __restrict__ m = mask + r0;
+  for (unsigned t = blockIdx.x * kWarps + w; t < T.count; t += gridDim.x * kWarps) {
+    unsigned row0, i0, cells;
+    T.tile(t, &row0, &i0, &cells);
+    const long long at0 = (long long)row0 * nx + i0;  // the tile's first cell
     int na = 0;
 #pragma unroll
     for (int s = 0; s < kTile / 32; ++s) {
-      const int i = i0 + 32 * s + lane;
-      const bool act = i < nx && m[i] > 0;
+      if (32 * s >= (int)cells) break;
+      const int c = 32 * s + lane;
+      const bool act = c < (int)cells && mask[at0 + c] > 0;
       const unsigned all = __ballot_sync(0xffffffffu, act);
-      if (act) active[w][na + __popc(all & ((1u << lane) - 1u))] = (uint8_t)(32 * s + lane);
+      if (act) active[w][na + __popc(all & ((1u << lane) - 1u))] = (uint8_t)c;
       na += __popc(all);
     }
     __syncwarp();
-    const bool row_in[4] = {j > 0, j + 1 < ny, k > 0, k + 1 < nz};
-    const double* __restrict__ fx = bx ? bx + (long long)row * (nx + 1) : nullptr;
-    const double* __restrict__ fy = by ? by + ((long long)k * (ny + 1) + j) * nx : nullptr;
-    const double* __restrict__ fz = bz ? bz + r0 : nullptr;
-    const double* __restrict__ p = phi + r0;
+    const int k0 = (int)(row0 / (unsigned)ny), j0 = (int)(row0 - (unsigned)k0 * (unsigned)ny);
     for (int x = lane; x < na; x += 32) {
-      const int i = i0 + active[w][x];
-      const bool in[6] = {i > 0 && m[i - 1] > 0,         i + 1 < nx && m[i + 1] > 0,    row_in[0] && m[i - sy] > 0,
-                          row_in[1] && m[i + sy] > 0,    row_in[2] && m[i - sz] > 0,    row_in[3] && m[i + sz] > 0};
+      const int c = active[w][x];
+      unsigned row = row0;
+      int i = (int)i0 + c, j = j0, k = k0;
+      if (ROWS) {
+        const unsigned dr = T.row_of((unsigned)c);
+        row += dr;
+        i = c - (int)dr * nx;
+        k = (int)(row / (unsigned)ny);
+        j = (int)(row - (unsigned)k * (unsigned)ny);
+      }
+      const int8_t* __restrict__ m = mask + (at0 + c);
+      const double* __restrict__ p = phi + (at0 + c);
+      const bool in[6] = {i > 0 && m[-1] > 0,      i + 1 < nx && m[1] > 0, j > 0 && m[-sy] > 0,
+                          j + 1 < ny && m[sy] > 0, k > 0 && m[-sz] > 0,    k + 1 < nz && m[sz] > 0};
       const long long off[6] = {-1, 1, -sy, sy, -sz, sz};
-      const double* f[6] = {fx ? fx + i : nullptr, fx ? fx + i + 1 : nullptr, fy ? fy + i : nullptr,
-                            fy ? fy + i + nx : nullptr, fz ? fz + i : nullptr, fz ? fz + i + sz : nullptr};
+      const long long fx = (long long)row * (nx + 1) + i, fy = (long long)(row + (unsigned)k) * nx + i, fz = at0 + c;
+      const double* f[6] = {bx ? bx + fx : nullptr,      bx ? bx + fx + 1 : nullptr, by ? by + fy : nullptr,
+                            by ? by + fy + nx : nullptr, bz ? bz + fz : nullptr,     bz ? bz + fz + sz : nullptr};
       double v[6];
       int ghosts = 0;
 #pragma unroll
       for (int d = 0; d < 6; ++d) {
         v[d] = 0.0;
-        if (in[d]) v[d] = p[i + off[d]];
+        if (in[d]) v[d] = p[off[d]];
         else if (f[d]) v[d] = twice(*f[d]);
         ghosts += !in[d];
       }
-      const double r = fma(-diag[ghosts], p[i], exact_sum(v)) - h2 * rho[r0 + i];
+      const double r = fma(-diag[ghosts], p[0], exact_sum(v)) - h2 * rho[at0 + c];
       acc = fma(r, r, acc);
     }
     __syncwarp();
@@ -186,16 +199,22 @@ extern "C" mg_status mg_residual_norm_noalloc(const int8_t* mask, const double* 
     set_thread_error("mg_residual_norm_noalloc: cudaGetSymbolAddress of the scratch array failed");
     return MG_ERR_CUDA;
   }
-  // a warp per tile of a row, at most the resident blocks
-  const long long tiles = (long long)((nx + kTile - 1) / kTile) * ny * nz;
-  long long blocks = (tiles + kNoAllocThreads / 32 - 1) / (kNoAllocThreads / 32);
-  if (blocks > (long long)kBlocksPerSm * device_sms()) blocks = (long long)kBlocksPerSm * device_sms();
+  // a warp per tile, at most the resident blocks
+  constexpr int kWarps = kNoAllocThreads / 32;
+  const int resident = kBlocksPerSm * device_sms();
+  const RowTiles T = row_tiles(nx, ny, nz, kTile, resident * kWarps);
+  long long blocks = ((long long)T.count + kWarps - 1) / kWarps;
+  if (blocks > resident) blocks = resident;
   if (blocks > kNoAllocMaxPartials) blocks = kNoAllocMaxPartials;
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const double h2 = h * h;
   count_launch(2);
-  noalloc_resnorm_kernel<<<(int)blocks, kNoAllocThreads, 0, s>>>(mask, phi, rho, bx, by, bz, nx, ny, nz, h2,
-                                                                  (double*)scratch);
+  if (T.per > 1)
+    noalloc_resnorm_kernel<true><<<(int)blocks, kNoAllocThreads, 0, s>>>(mask, phi, rho, bx, by, bz, T, ny, nz, h2,
+                                                                         (double*)scratch);
+  else
+    noalloc_resnorm_kernel<false><<<(int)blocks, kNoAllocThreads, 0, s>>>(mask, phi, rho, bx, by, bz, T, ny, nz, h2,
+                                                                          (double*)scratch);
   noalloc_finalize_kernel<<<1, kNoAllocThreads, 0, s>>>((const double*)scratch, (int)blocks, h2, norm_out);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

@@ -1,0 +1,75 @@
+"""The residual norm from caller buffers on boxes with short rows, where a tile
+takes several of them: rows of one cell up to the longest that two fit a tile, a
+last tile that is not full, against the residual by plain torch in the same
+precision (six additions and two multiplications per cell, relative error of a
+norm far below 1e-12); and non-finite values at active cells and none from
+inactive ones."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1104_1703_gb300 import binding as B  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+# (nz, ny, nx): more rows than the GPU holds warps, down to few
+SHAPES = [(1024, 512, 1), (101, 151, 1), (300, 211, 2), (200, 300, 3), (512, 512, 5), (256, 257, 16), (130, 129, 33),
+          (150, 150, 85), (128, 128, 127), (128, 129, 128), (5, 7, 9), (1, 1, 1), (2048, 3, 2), (3, 2048, 7)]
+
+
+def _fields(shape, seed, p_active):
+    nz, ny, nx = shape
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    draw = lambda s: torch.randn(s, generator=g, device="cuda", dtype=torch.float64)  # noqa: E731
+    mask = (torch.rand(shape, generator=g, device="cuda") < p_active).to(torch.int8)
+    mask[0, 0, 0] = 1
+    return mask, draw(shape), draw(shape), [draw(s) for s in ((nz, ny, nx + 1), (nz, ny + 1, nx), (nz + 1, ny, nx))]
+
+
+def reference(mask, phi, rho, h, faces):
+    act = mask > 0
+    a = torch.where(act, phi, torch.zeros_like(phi))
+    r = -h * h * rho
+    diag = torch.full_like(phi, 6.0)
+    for axis in range(3):
+        n = phi.shape[axis]
+        for step in (-1, 1):
+            inside = torch.zeros_like(act)
+            near = torch.zeros_like(a)
+            to, src = (slice(1, n), slice(0, n - 1)) if step < 0 else (slice(0, n - 1), slice(1, n))
+            ix = lambda s: tuple(s if d == axis else slice(None) for d in range(3))  # noqa: E731
+            inside[ix(to)] = act[ix(src)]
+            near[ix(to)] = a[ix(src)]
+            face = faces[2 - axis].narrow(axis, 0 if step < 0 else 1, n)
+            r = r + torch.where(inside, near, 2.0 * face)
+            diag = diag + (~inside).double()
+    r = torch.where(act, r - diag * a, torch.zeros_like(a))
+    return float((r.square().sum().sqrt() / (h * h)).item())
+
+
+def norm(mask, phi, rho, h, faces):
+    out = torch.zeros(1, dtype=torch.float64, device="cuda")
+    B.mg_residual_norm_noalloc(mask, phi, rho, h, out, *faces)
+    return float(out.item())
+
+
+@pytest.mark.parametrize("p_active", [0.03, 0.6, 1.0])
+@pytest.mark.parametrize("shape", SHAPES)
+def test_norm(shape, p_active):
+    mask, phi, rho, faces = _fields(shape, 11, p_active)
+    phi = torch.where(mask > 0, phi, torch.full_like(phi, float("nan")))  # inactive cells are ignored
+    rho = torch.where(mask > 0, rho, torch.full_like(rho, float("inf")))
+    want = reference(mask, phi, torch.where(mask > 0, rho, torch.zeros_like(rho)), 0.125, faces)
+    assert abs(norm(mask, phi, rho, 0.125, faces) - want) <= 1e-12 * want
+
+
+@pytest.mark.parametrize("shape", [(200, 300, 3), (40, 40, 200)])
+@pytest.mark.parametrize("value", [float("inf"), -float("inf"), float("nan"), 1e200])
+@pytest.mark.parametrize("where", ["phi", "rho", "face"])
+def test_non_finite(shape, value, where):
+    mask, phi, rho, faces = _fields(shape, 12, 1.0)
+    {"phi": phi, "rho": rho, "face": faces[0]}[where][shape[0] // 2, shape[1] // 3, 0] = value
+    want, got = reference(mask, phi, rho, 0.125, faces), norm(mask, phi, rho, 0.125, faces)
+    assert not np.isfinite(want) and np.array_equal(got, want, equal_nan=True)
