@@ -15,6 +15,7 @@
 //  - Section 1 / Fig. 1: the fine Dirichlet values sit on the boundary faces
 //    and come from the coarser AMR level by linear interpolation.
 #include "mg_internal.h"
+#include "row_tiles.h"
 
 namespace gbmg {
 
@@ -306,35 +307,51 @@ __device__ __forceinline__ void face_centre2(int d, int i, int j, int k, int& x2
 // Only the FP64 pipe (2 lanes per clock and SM, idle lanes included) bounds
 // it: about 17 operations per face, and a thread per cell ran them for every
 // direction in every warp (320 us on a half-active 128^3 blob patch).  So a
-// warp takes 128 cells of a row at a time, lists their ghost faces and their
-// boundary cells, and works through both lists with every lane in use; the
-// other cells only copy h^2 rho.
+// warp takes 128 cells of a row, or of several short rows (row_tiles.h), at a
+// time, lists their ghost faces and their boundary cells, and works through
+// both lists with every lane in use; the other cells only copy h^2 rho.
+// Short rows (the whole call, half-active boxes): 512 x 512 rows of 8 cells 151
+// us, 412 with a tile per row, 872 with a thread per cell; 1024 x 1024 rows of
+// one cell 154, 875 and 552.
 constexpr int kFoldWarps = 4;
 constexpr int kFoldCells = 128;
+constexpr int kFoldBlocks = 6;  // per SM, by their shared memory
 
+template <bool ROWS>
 __global__ void __launch_bounds__(32 * kFoldWarps)
-    fold_coarse_kernel(LevelDev L, FineExtra F, const double* __restrict__ pc, int cnx, int cny, int cnz, int ox,
-                       int oy, int oz, int* err_flag) {
+    fold_coarse_kernel(LevelDev L, FineExtra F, RowTiles T, const double* __restrict__ pc, int cnx, int cny, int cnz,
+                       int ox, int oy, int oz, int* err_flag) {
   __shared__ double vals[kFoldWarps][6 * kFoldCells];
   __shared__ uint16_t faces[kFoldWarps][6 * kFoldCells];     // cell | direction << 8
   __shared__ uint16_t cells[kFoldWarps][kFoldCells];         // boundary cells of the tile
   __shared__ uint16_t start[kFoldWarps][kFoldCells + 1];     // their first face
   const Geom g = L.g;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const unsigned tiles = (unsigned)(g.nx + kFoldCells - 1) / kFoldCells;
-  const unsigned n = tiles * (unsigned)g.ny * (unsigned)g.nz;
-  for (unsigned t = blockIdx.x * kFoldWarps + w; t < n; t += gridDim.x * kFoldWarps) {
-    const unsigned row = t / tiles;
-    const int k = (int)(row / (unsigned)g.ny), j = (int)(row - (unsigned)k * (unsigned)g.ny);
-    const int i0 = (int)(t - row * tiles) * kFoldCells;
-    const long long base = g.at(0, j, k);
+  for (unsigned t = blockIdx.x * kFoldWarps + w; t < T.count; t += gridDim.x * kFoldWarps) {
+    unsigned row0, i0, ncell;
+    T.tile(t, &row0, &i0, &ncell);
+    const int k0 = (int)(row0 / (unsigned)g.ny), j0 = (int)(row0 - (unsigned)k0 * (unsigned)g.ny);
+    // place of the tile's cell
+    auto place = [&](int cell, int& i, int& j, int& k) {
+      i = (int)i0 + cell;
+      j = j0;
+      k = k0;
+      if (ROWS) {
+        const unsigned dr = T.row_of((unsigned)cell);
+        i = cell - (int)(dr * T.nx);
+        k = (int)((row0 + dr) / (unsigned)g.ny);
+        j = (int)(row0 + dr - (unsigned)k * (unsigned)g.ny);
+      }
+    };
     int nf = 0, nc = 0;
 #pragma unroll
     for (int s = 0; s < kFoldCells / 32; ++s) {
-      const int i = i0 + 32 * s + lane;
-      const bool in = i < g.nx;
+      if (32 * s >= (int)ncell) break;
+      const bool in = 32 * s + lane < (int)ncell;
+      int i, j, k;
+      place(in ? 32 * s + lane : 0, i, j, k);
       const int c = colour_of(i, j, k);
-      const long long at = base + (i >> 1);
+      const long long at = g.at(i >> 1, j, k);
       const uint8_t code = in ? L.code[c][at] : 0;
       const int gh = (code & kActive2) ? code >> kGhostShift : 0;
       const int cnt = __popc(gh);
@@ -362,17 +379,19 @@ __global__ void __launch_bounds__(32 * kFoldWarps)
     __syncwarp();
     for (int x = lane; x < nf; x += 32) {
       const int e = faces[w][x];
-      int x2, y2, z2;
-      face_centre2(e >> 8, i0 + (e & 255), j, k, x2, y2, z2);
+      int i, j, k, x2, y2, z2;
+      place(e & 255, i, j, k);
+      face_centre2(e >> 8, i, j, k, x2, y2, z2);
       double v = 0.0;
       if (!coarse_sample(pc, cnx, cny, cnz, ox, oy, oz, x2, y2, z2, v)) atomicExch(err_flag, 1);
       vals[w][x] = v;
     }
     __syncwarp();
     for (int x = lane; x < nc; x += 32) {
-      const int i = i0 + cells[w][x];
+      int i, j, k;
+      place(cells[w][x], i, j, k);
       const int c = colour_of(i, j, k);
-      const long long at = base + (i >> 1);
+      const long long at = g.at(i >> 1, j, k);
       double acc = 0.0;
       for (int f = start[w][x]; f < start[w][x + 1]; ++f) acc += vals[w][f];
       const double bc = 2.0 * acc;
@@ -697,11 +716,13 @@ cudaError_t launch_fold_faces(const LevelDev& L0, const FineExtra& F, const doub
 cudaError_t launch_fold_coarse(const LevelDev& L0, const FineExtra& F, const double* pc, int cnx, int cny,
                                int cnz, int ox, int oy, int oz, int* err_flag, cudaStream_t s) {
   count_launch();
-  const long long tiles = (long long)((L0.g.nx + kFoldCells - 1) / kFoldCells) * L0.g.ny * L0.g.nz;
-  long long blocks = (tiles + kFoldWarps - 1) / kFoldWarps;
+  const int resident = kFoldBlocks * device_sms();
+  const RowTiles T = row_tiles(L0.g.nx, L0.g.ny, L0.g.nz, kFoldCells, resident * kFoldWarps);
+  long long blocks = ((long long)T.count + kFoldWarps - 1) / kFoldWarps;
   if (blocks > 32LL * device_sms()) blocks = 32LL * device_sms();
-  fold_coarse_kernel<<<(int)blocks, 32 * kFoldWarps, 0, s>>>(L0, F, pc, cnx, cny, cnz, clamp_origin(ox), clamp_origin(oy),
-                                                          clamp_origin(oz), err_flag);
+  auto kernel = T.per > 1 ? fold_coarse_kernel<true> : fold_coarse_kernel<false>;
+  kernel<<<(int)blocks, 32 * kFoldWarps, 0, s>>>(L0, F, T, pc, cnx, cny, cnz, clamp_origin(ox), clamp_origin(oy),
+                                                 clamp_origin(oz), err_flag);
   return cudaGetLastError();
 }
 

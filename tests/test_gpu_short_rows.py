@@ -1,9 +1,9 @@
-"""The residual norm from caller buffers on boxes with short rows, where a tile
-takes several of them: rows of one cell up to the longest that two fit a tile, a
-last tile that is not full, against the residual by plain torch in the same
-precision (six additions and two multiplications per cell, relative error of a
-norm far below 1e-12); and non-finite values at active cells and none from
-inactive ones."""
+"""The residual norm from caller buffers and the fold of the coarser level's values
+on boxes with short rows, where a tile takes several of them: rows of one cell
+up to the longest that two fit a tile, a last tile that is not full.  The norm
+against the residual by plain torch in the same precision (six additions and two
+multiplications per cell, relative error of a norm far below 1e-12), with
+non-finite values at active cells and none taken from inactive ones."""
 import numpy as np
 import pytest
 
@@ -73,3 +73,26 @@ def test_non_finite(shape, value, where):
     {"phi": phi, "rho": rho, "face": faces[0]}[where][shape[0] // 2, shape[1] // 3, 0] = value
     want, got = reference(mask, phi, rho, 0.125, faces), norm(mask, phi, rho, 0.125, faces)
     assert not np.isfinite(want) and np.array_equal(got, want, equal_nan=True)
+
+
+@pytest.mark.parametrize("p_active", [0.03, 0.6, 1.0])
+@pytest.mark.parametrize("shape", [s for s in SHAPES if s[2] < 128] + [(100, 111, 63), (90, 100, 64), (90, 100, 65)])
+def test_fold(shape, p_active):
+    """Boundary values interpolated from the coarser level and folded, against the same values as face arrays."""
+    nz, ny, nx = shape
+    mask, rho, _, faces = _fields(shape, 13, p_active)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(14)
+    phi_c = torch.randn(tuple((n + 1) // 2 + 2 for n in shape), generator=g, device="cuda", dtype=torch.float64)
+    with B.Hierarchy(mask, 0.125) as H:
+        H.set_rhs(rho)
+        H.set_dirichlet_from_coarse(phi_c, (-2, -2, -2))
+        got = H.level_get(0, B.MG_FIELD_RHS)
+        H.faces_from_coarse(phi_c, (-2, -2, -2), *faces)
+        H.set_dirichlet(*faces)
+        want = H.level_get(0, B.MG_FIELD_RHS)
+        if p_active == 1.0:
+            with pytest.raises(B.MGError):
+                H.set_dirichlet_from_coarse(phi_c, (-2, 0, -2))
+    # the same six terms added in another order at most: 6 roundings of values below 12 max|phi_c|
+    assert np.abs(got - want).max() <= 6 * 2.0 ** -52 * 12 * float(phi_c.abs().max())
