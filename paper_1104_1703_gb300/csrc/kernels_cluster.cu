@@ -261,6 +261,52 @@ struct ClArgs {
   } deep[kClMaxLevels];
 };
 
+// Sweeps of a level of the tail, which CTA 0 runs alone: nothing is sent, one
+// record per colour and thread, all that stays fixed in registers.  Its own loop,
+// because the deepest level often takes 2 * coarse_sweeps half-sweeps here (no
+// map above kCoarseMatMax unknowns): in the loop of the distributed levels, which
+// holds two records and the sends, each cost 0.2 to 0.3 us more (FP64: every
+// idle slot's instructions take the FP64 pipe), 15 to 30 us per visit.  V-cycles
+// (launch per step; that loop; this one): 161 x 200 x 143 with holes, first order,
+// 346 unknowns deepest, FP64 401, 419, 398 us, FP32 132, 142, 123; 96 x 80 x 100,
+// 68 unknowns, FP64 181, 169, 139.  (One warp for levels of at most 64 unknowns
+// per colour, two records per thread: 163 in the last.)
+template <int KIND, typename T>
+__device__ __forceinline__ void cl_tail_sweeps(T* const (&phi)[2], const uint16_t* const (&off)[2],
+                                               const T* const (&b)[2], const T* const (&id)[2], const uint32_t (&n)[2],
+                                               int Ps, int pl, int sweeps) {
+  const uint32_t x = threadIdx.x;
+  bool has[2];
+  T* self[2];
+  const T* other[2];
+  int dx[2];
+  T bb[2], ii[2];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    has[c] = x < n[c];
+    const uint32_t e = has[c] ? off[c][x] : 0u;
+#ifdef MG_CHECKED
+    has[c] = has[c] && (e & 0x7fffu) != 0;  // an entry that failed its bounds check
+#endif
+    self[c] = phi[c] + (e & 0x7fffu);
+    other[c] = phi[c ^ 1] + (e & 0x7fffu);
+    dx[c] = (e & 0x8000u) ? 1 : -1;
+    bb[c] = has[c] ? b[c][x] : T(0);
+    ii[c] = KIND == 1 ? (has[c] ? id[c][x] : T(0)) : T(1) / T(6);
+  }
+#pragma unroll 1
+  for (int s = 0; s < sweeps; ++s)
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      if (has[c]) {
+        const T* p = other[c];
+        const T sum = ((p[0] + p[dx[c]]) + (p[-Ps] + p[Ps])) + (p[-pl] + p[pl]);
+        *self[c] = (sum - bb[c]) * ii[c];
+      }
+      __syncthreads();
+    }
+}
+
 template <int KIND, typename T>
 __global__ void __launch_bounds__(kClThreads, 1) cluster_cycle_kernel(const __grid_constant__ ClArgs<T> a) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -439,24 +485,26 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_cycle_kernel(const __gr
         }
       }
       __syncthreads();
+    } else if (i >= a.tail) {
+      T* const f[2] = {arr(phi[0]), arr(phi[1])};
+      const uint16_t* const off[2] = {u16(hoff[0]), u16(hoff[1])};
+      const T* const b[2] = {arr(hb[0]), arr(hb[1])};
+      const T* const id[2] = {arr(hid[0]), arr(hid[1])};
+      cl_tail_sweeps<KIND, T>(f, off, b, id, n, Ps, pl, sweeps);
     } else {
       const Exchange ex[2] = {exchange(h, 0), exchange(h, 1)};
       const uint32_t lo_end = (h.flags & 1u) ? h.lo_end : 0u, hi_begin = (h.flags & 2u) ? h.hi_begin : 0xffffffffu;
       const uint32_t lo_to[2] = {lo_base + h.lo[0], lo_base + h.lo[1]}, hi_to[2] = {hi_base + h.hi[0], hi_base + h.hi[1]};
       if (n[0] <= (uint32_t)(kClHoist * kClThreads) && n[1] <= (uint32_t)(kClHoist * kClThreads)) {
         // what stays fixed over the sweeps in registers, so a half-sweep is
-        // six loads per record, the update, its store and the exchange; a
-        // level of CTA 0 with at most 64 unknowns per colour is swept by warp
-        // 0 alone
-        const bool one_warp = i >= a.tail && n[0] <= 32 * kClHoist && n[1] <= 32 * kClHoist;
-        const uint32_t nthr = one_warp ? 32u : (uint32_t)kClThreads;
+        // six loads per record, the update, its store and the exchange
         uint32_t at[2][kClHoist];  // element offset; bit 15: x-neighbour, 16: present, 17 / 18: goes to the lower / upper CTA
         T bb[2][kClHoist], ii[2][kClHoist];
 #pragma unroll
         for (int c = 0; c < 2; ++c)
 #pragma unroll
           for (int k = 0; k < kClHoist; ++k) {
-            const uint32_t x = tid + k * nthr;
+            const uint32_t x = tid + k * kClThreads;
             bool has = x < n[c];
             uint32_t e = has ? u16(hoff[c])[x] : 0u;
 #ifdef MG_CHECKED
@@ -467,33 +515,29 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_cycle_kernel(const __gr
             const uint32_t o = e & 0x7fffu;
             at[c][k] = e | (has ? 1u << 16 : 0u) | (has && o < lo_end ? 1u << 17 : 0u) | (has && o >= hi_begin ? 1u << 18 : 0u);
           }
-        if (!one_warp || tid < 32) {
 #pragma unroll 1
-          for (int s = 0; s < sweeps; ++s) {
+        for (int s = 0; s < sweeps; ++s) {
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-              T v[kClHoist];
+          for (int c = 0; c < 2; ++c) {
+            T v[kClHoist];
 #pragma unroll
-              for (int k = 0; k < kClHoist; ++k) {
-                if (!(at[c][k] & (1u << 16))) continue;
-                const T* p = arr(phi[c ^ 1]) + (at[c][k] & 0x7fffu);
-                const T sum = ((p[0] + p[(at[c][k] & 0x8000u) ? 1 : -1]) + (p[-Ps] + p[Ps])) + (p[-pl] + p[pl]);
-                v[k] = (sum - bb[c][k]) * ii[c][k];
-              }
-#pragma unroll
-              for (int k = 0; k < kClHoist; ++k) {
-                if (!(at[c][k] & (1u << 16))) continue;
-                const uint32_t o = phi[c] + (at[c][k] & 0x7fffu) * W;
-                *arr(o) = v[k];
-                if (at[c][k] & (1u << 17)) st_async(lo_to[c] + o, v[k], lo_bar + 8u * c);
-                if (at[c][k] & (1u << 18)) st_async(hi_to[c] + o, v[k], hi_bar + 8u * c);
-              }
-              if (one_warp) __syncwarp();
-              else settle(ex[c], c);
+            for (int k = 0; k < kClHoist; ++k) {
+              if (!(at[c][k] & (1u << 16))) continue;
+              const T* p = arr(phi[c ^ 1]) + (at[c][k] & 0x7fffu);
+              const T sum = ((p[0] + p[(at[c][k] & 0x8000u) ? 1 : -1]) + (p[-Ps] + p[Ps])) + (p[-pl] + p[pl]);
+              v[k] = (sum - bb[c][k]) * ii[c][k];
             }
+#pragma unroll
+            for (int k = 0; k < kClHoist; ++k) {
+              if (!(at[c][k] & (1u << 16))) continue;
+              const uint32_t o = phi[c] + (at[c][k] & 0x7fffu) * W;
+              *arr(o) = v[k];
+              if (at[c][k] & (1u << 17)) st_async(lo_to[c] + o, v[k], lo_bar + 8u * c);
+              if (at[c][k] & (1u << 18)) st_async(hi_to[c] + o, v[k], hi_bar + 8u * c);
+            }
+            settle(ex[c], c);
           }
         }
-        if (one_warp) __syncthreads();
       } else {
 #pragma unroll 1
         for (int half = 0; half < 2 * sweeps; ++half) {
@@ -718,7 +762,9 @@ long long level_slots(const Geom& g) { return (long long)g.hx * g.ny * g.nz; }
 // launch on all of them (3.6 us), and above 256 the tail's costs more than an
 // exchange (600 cycles).  FP32: about 0.45 cycles per unknown.
 uint32_t cl_max_unknowns(int prec) { return prec == kFP64 ? 1280u : 8192u; }
-uint32_t cl_max_tail(int prec) { return prec == kFP64 ? 256u : 256u; }
+bool cl_tail_level(const LevelDev& D, int order) {
+  return D.hcount[order * 2] <= (uint32_t)kClThreads && D.hcount[order * 2 + 1] <= (uint32_t)kClThreads;
+}
 
 template <typename T>
 struct ClFields {
@@ -798,12 +844,10 @@ bool cl_plan_from(const LevelDev* levels, int m, int deepest, int order, int pre
   p.nlev = deepest - m + 1;
   if (m < 1 || p.nlev < 1 || p.nlev > kClMaxLevels) return false;
   p.first = m;
-  while (p.tail < p.nlev) {
-    const LevelDev& D = levels[m + p.tail];
-    if (!D.hpstart[order][0]) return false;
-    if (D.hcount[order * 2] <= cl_max_tail(prec) && D.hcount[order * 2 + 1] <= cl_max_tail(prec)) break;
-    ++p.tail;
-  }
+  // the tail: from its first level on all are small (a coarser level never has
+  // more unknowns, but it can have more of one colour)
+  p.tail = p.nlev;
+  while (p.tail > 0 && cl_tail_level(levels[m + p.tail - 1], order)) --p.tail;
   if (p.tail == 0) return false;  // one CTA: the bottom cycle's case
   const int nzc = levels[m + p.tail - 1].g.nz;
   if (nzc < 2) return false;
