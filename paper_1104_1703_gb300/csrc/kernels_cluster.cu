@@ -3,18 +3,19 @@
 // arXiv:1104.1703, Section 2 recipe on levels m .. deepest).
 //
 // What bounds these levels: 10^2 to 10^5 unknowns are too few to fill the
-// GPU, so a launch per step costs its latency (3.0 to 3.9 us per half-sweep
-// of a 64^3 or 32^3 level, whatever it holds), and one CTA alone is bound by
-// its SM's FP64 rate (2 operations per clock) on a 16^3 level.  Here the
-// levels live in the shared memory of up to 16 SMs for the whole visit.
+// GPU, so a launch per step costs its latency (1.65 to 2.0 us per half-sweep of
+// a 64^3 or 32^3 level in a replayed graph, whatever it holds), and one CTA alone
+// is bound by its SM's FP64 rate (2 operations per clock) on a 16^3 level.  Here
+// the levels live in the shared memory of up to 16 SMs for the whole visit: a
+// half-sweep with its exchange takes 0.32 (FP32) to 0.6 us (FP64).
 //
 // Split.  A level is cut into slabs of z-planes, one per CTA; the cut of the
 // coarsest distributed level decides (so that the fullest CTA holds as few
 // unknowns as the shared memory allows) and every finer cut is its double, so
 // the children of a CTA's cells are its own.  The levels below (the tail)
 // belong to CTA 0 alone, which runs them with block barriers while the others
-// wait: an exchange costs 500 to 700 cycles, so a level is distributed only
-// when one SM would take longer.  Per level a CTA holds
+// wait (0.06 to 0.1 us per half-sweep in FP32, 0.27 to 0.45 in FP64): a level is
+// distributed only when one SM would take longer.  Per level a CTA holds
 //  - its correction dPhi, dense, both colours, with one halo row in y, one
 //    padding slot per row and one halo plane on each side in z;
 //  - its unknowns as records in list order: a 16-bit offset (bit 15: the
@@ -756,12 +757,24 @@ __global__ void __launch_bounds__(kClThreads, 1) cluster_cycle_kernel(const __gr
 
 long long level_slots(const Geom& g) { return (long long)g.hx * g.ny * g.nz; }
 
-// Most unknowns of one colour that a CTA takes of a distributed level, and
-// that the tail's one CTA takes.  FP64: an SM retires 2 operations per clock,
-// 7 per unknown, so above 1280 a half-sweep on 16 SMs costs more than its own
-// launch on all of them (3.6 us), and above 256 the tail's costs more than an
-// exchange (600 cycles).  FP32: about 0.45 cycles per unknown.
-uint32_t cl_max_unknowns(int prec) { return prec == kFP64 ? 1280u : 8192u; }
+// Most unknowns of one colour that a CTA takes of a distributed level; a level
+// above it runs as one launch per step on all SMs.  Measured per V-cycle of the
+// whole hierarchy (12 in one graph), with that level in the cluster and without:
+//  - FP64, bound by the FP64 pipe of 16 SMs: 427 to 512 per CTA gain (150 x 15 x
+//    15 72.7 -> 68.5 us, 256 x 8 x 8 67.0 -> 64.7), 550 to 1152 lose (29 x 22 x
+//    31 61.7 -> 69.0, 32^3 of a ball 65.7 -> 73.2, all of 32^3 82.5 -> 94.4, 24^3
+//    69.1 -> 90.6);
+//  - FP64 levels that the one-CTA bottom takes otherwise (small_level): 20^3, 800
+//    per CTA, 148 -> 76; 3 x 32 x 32, 1024, 94 -> 89;
+//  - FP32: up to 2048 per CTA gain (24^3, 1152, 48.9 -> 45.3; 32^3, 1024, 51.3 ->
+//    47.0; 8 x 8 x 256, 2048, 45.4 -> 44.2), from 2250 on they lose (15 x 150 x
+//    15 49.7 -> 51.5, 64^3 of a union, 3307, 136.9 -> 143.9, 36^3, 5184, 55.7 ->
+//    71.2).
+uint32_t cl_max_unknowns(const LevelDev& D, int prec) {
+  if (prec == kFP32) return 2048u;
+  return small_level(D.g) ? 1280u : 512u;
+}
+// The tail's levels: one record per colour and thread of its one CTA.
 bool cl_tail_level(const LevelDev& D, int order) {
   return D.hcount[order * 2] <= (uint32_t)kClThreads && D.hcount[order * 2 + 1] <= (uint32_t)kClThreads;
 }
@@ -878,7 +891,7 @@ bool cl_plan_from(const LevelDev* levels, int m, int deepest, int order, int pre
     }
     if (i >= p.tail) tail_bytes += t.plane * (t.nz + 2);
   }
-  const uint32_t cap = cl_max_unknowns(prec);
+  const uint32_t cap = cl_max_unknowns(levels[m], prec);
   if (total > (uint64_t)cap * p.ranks) return false;
   auto fits = [&](int r, int zc0, int zc1, uint32_t most) {
     size_t bytes = fixed + (r == 0 ? tail_bytes : 0);
@@ -1110,8 +1123,10 @@ size_t cluster_blob_bound(const LevelDev* levels, int nlev, int prec) {
 
 ClPlan cluster_plan(const LevelDev* levels, int deepest, int order, int prec, size_t blob_bound) {
   ClPlan p;
-  for (int m = 1; m <= deepest; ++m)
+  for (int m = 1; m <= deepest; ++m) {
     if (cl_plan_from(levels, m, deepest, order, prec, p) && (size_t)p.stride * p.ranks <= blob_bound) return p;
+    if (small_level(levels[m].g)) break;  // the one-CTA bottom takes everything from here on
+  }
   return ClPlan();
 }
 
