@@ -583,6 +583,21 @@ bool capture_loop(mg_hierarchy* H, int order, GraphSlot& gs) {
   return gs.exec != nullptr;
 }
 
+// Whether a solve from relative residual rel to tol runs its cycles in the loop.
+// Its launch costs 15 us more than a single cycle's (the state's copies, the
+// node), each of its iterations 4 less: from about four cycles on it pays.  A
+// multigrid iteration gains about a decade (mixed form: inner_cycles of them per
+// cycle); a hierarchy of one level, which only sweeps, and a line of cells, which
+// the coarse correction solves exactly, end in one or two.  (4^3 ball, FP64, one
+// cycle: 123 us, 146 in the loop; 16^3, mixed, 4 inner cycles, two steps: 384,
+// 405; 32^3 ball, FP64, 9 cycles: 805, 783.)
+bool loop_pays(const mg_hierarchy* H, int order, double rel, double tol) {
+  const Geom& g = H->L[0].g;
+  if (H->deepest[order] == 0 || g.ncells() == std::max({g.nx, g.ny, g.nz})) return false;
+  const int inner = H->opt.precision == 1 ? H->opt.inner_cycles : 1;
+  return std::log10(rel / tol) >= 4.0 * inner;
+}
+
 // Up to `budget` cycles of `order` in one launch, as long as the state's rule
 // asks for another; their norms are left in H->hloop.  *ran = false: this
 // hierarchy does not loop on the device.
@@ -1433,8 +1448,9 @@ mg_status mg_solve(mg_hierarchy* H, double tol, int max_cycles, mg_solve_info* i
     const int inner = o.precision == 1 ? o.inner_cycles : 1;
     const double eta_step = std::pow(o.eta, (double)inner);
     int ahead = 0, looked = 0;  // cycles the device has done and those of them looked at here
+    const bool in_loop = loop_pays(H, order, rel, tol);
     for (cycles = 1; cycles <= max_cycles; ++cycles) {
-      if (looked == ahead) {
+      if (in_loop && looked == ahead) {
         CycleLoop& lp = *H->hloop;
         lp.h2 = H->h * H->h;
         lp.r_zero = r_zero;
