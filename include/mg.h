@@ -93,8 +93,9 @@ typedef enum { MG_MEM_HOST = 0, MG_MEM_DEVICE = 1 } mg_mem;
  *                  one thread-block cluster, through global memory; 0 = the
  *                  coarse levels that fit the shared memory of a cluster run
  *                  from there as one launch (n_pre, n_post >= 1), the ones
- *                  above them one launch per step (faster on GB300).  The
- *                  results are the same.
+ *                  above them one launch per step (faster on GB300; their
+ *                  records take at most 3.7 MB per order).  The results are
+ *                  the same.
  *  smoother_pass   mixed form: 1 = run each pair of FP32 Gauss-Seidel sweeps
  *                  of the fine level (N_pre = N_post = 2 is one pair) as one
  *                  temporal-blocked pass over the level (a z-wavefront over
@@ -420,7 +421,10 @@ mg_status mg_batch_destroy(mg_batch* batch);
 
 /* The hierarchy of patch p, owned by the batch (do not destroy it).  Its
  * right-hand side, Dirichlet values and initial guess are set, and its
- * solution read, with the mg_hierarchy calls above.  Errors: INVALID_ARG. */
+ * solution read, with the mg_hierarchy calls above.  mg_solve and mg_vcycle on
+ * it work too; the first of them allocates the records of the coarse levels'
+ * cluster launch (option coarse_cluster), which batched cycles do not use, and
+ * runs without them if the device is full.  Errors: INVALID_ARG. */
 mg_status mg_batch_patch(mg_batch* batch, int p, mg_hierarchy** out);
 
 /* One multigrid iteration of every patch in its current order (as

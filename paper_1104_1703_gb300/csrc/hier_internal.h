@@ -88,10 +88,13 @@ struct mg_hierarchy {
   // the coarse levels' cluster launch per order (first level 0: none) and its
   // record blobs, and a hash of the list lengths and plane starts (captured
   // graphs depend on them)
-  bool cluster_ok = false;
+  bool patch = false;       // of a batch
+  bool cluster_ok = false;  // the device runs the largest cluster
+  bool cl_stale = true;     // the mask changed since the plans were made
   gbmg::ClPlan cl_plan[3];
   char* cl_blobs[3] = {nullptr, nullptr, nullptr};
-  size_t cl_bound = 0;
+  size_t cl_bound = 0;      // bytes of each
+  char* cl_own = nullptr;   // a patch's records, outside the arena
   unsigned long long lists_hash = 0;
   double* hscal = nullptr;               // pinned host scalars
   void* staging = nullptr;
@@ -115,5 +118,9 @@ struct mg_hierarchy {
 };
 
 namespace gbmg {
-mg_status check_faults(mg_hierarchy* H);  // mg_capi.cu
+// mg_capi.cu
+mg_status check_faults(mg_hierarchy* H);
+// mg_create_hierarchy; patch: for a batch, whose own cycles run its coarse levels
+mg_status create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, int nz, double h, const mg_options* opt,
+                           void* cuda_stream, bool patch, mg_hierarchy** out);
 }  // namespace gbmg

@@ -669,7 +669,7 @@ mg_status mg_batch_create(int n_patches, const int8_t* const* masks, mg_mem wher
   B->P.assign(n_patches, nullptr);
   for (int p = 0; p < n_patches && st == MG_OK; ++p) {
     mg_hierarchy* H = nullptr;
-    st = mg_create_hierarchy(masks[p], where, dims[3 * p], dims[3 * p + 1], dims[3 * p + 2], h[p], &o, B->stream, &H);
+    st = create_hierarchy(masks[p], where, dims[3 * p], dims[3 * p + 1], dims[3 * p + 2], h[p], &o, B->stream, true, &H);
     if (st != MG_OK) {
       std::string msg = "patch " + std::to_string(p) + ": " + mg_last_error(nullptr);
       st = bfail(B, st, msg);

@@ -439,6 +439,33 @@ void drop_graph(GraphSlot& g) {
   g.deepest = -2;
 }
 
+// Plans and records of the coarse levels' cluster launches, for the current
+// mask.  A patch of a batch, whose batched cycles never launch them, allocates
+// the records' memory here, with its first own cycle; without it (the device is
+// full) the cycle runs launch by launch.
+mg_status build_cluster(mg_hierarchy* H) {
+  if (!H->cl_stale || !cluster_runs(H)) return MG_OK;
+  const int prec = H->opt.precision == 1 ? kFP32 : kFP64;
+  if (H->patch && !H->cl_own && H->cl_bound == 0) {
+    H->cl_bound = cluster_blob_bound(H->L, H->nlev, prec);
+    if (H->cl_bound && dev_malloc((void**)&H->cl_own, 2 * H->cl_bound) != cudaSuccess) {
+      (void)cudaGetLastError();
+      H->cl_own = nullptr;
+    }
+    for (int o = 1; o <= 2 && H->cl_own; ++o) H->cl_blobs[o] = H->cl_own + (o - 1) * H->cl_bound;
+  }
+  for (int o = 1; o <= 2; ++o) {
+    H->cl_plan[o] = ClPlan();
+    if (!H->cl_blobs[o]) continue;
+    H->cl_plan[o] = cluster_plan(H->L, H->deepest[o], o, prec, H->cl_bound);
+    if (H->cl_plan[o].first)
+      CKS(launch_ok(H, launch_cluster_build(H->L, H->cl_plan[o], o, prec, H->cl_blobs[o], H->stream),
+                    "coarse-level records"));
+  }
+  H->cl_stale = false;
+  return MG_OK;
+}
+
 // What a captured cycle depends on besides the hierarchy's fixed options:
 // noted at its capture, and compared before it is replayed.
 void note_key(const mg_hierarchy* H, int order, GraphSlot& g) {
@@ -604,6 +631,7 @@ bool loop_pays(const mg_hierarchy* H, int order, double rel, double tol) {
 mg_status run_loop(mg_hierarchy* H, int order, int budget, bool* ran) {
   *ran = false;
   if (!H->loop_ok || !H->opt.use_graphs || H->timing || H->pass_on) return MG_OK;
+  CKS(build_cluster(H));
   CKS(ensure_rhsd(H));
   if (H->opt.precision == 1 && !H->prepared) CKS(emit_refine_residual(H));
   H->prepared = true;
@@ -631,6 +659,7 @@ mg_status check_coarse_wait(mg_hierarchy* H, double r) {
 }
 
 mg_status run_cycle(mg_hierarchy* H, int order, double* r_out) {
+  CKS(build_cluster(H));
   CKS(ensure_rhsd(H));
   if (H->opt.precision == 1 && !H->prepared) CKS(emit_refine_residual(H));
   H->prepared = true;
@@ -731,15 +760,10 @@ mg_status build_levels(mg_hierarchy* H, bool fine_built = false, const int8_t* m
     H->deepest[o] = -1;
     for (int l = 0; l < H->nlev && H->active[o][l] > 0; ++l) H->deepest[o] = l;
   }
-  // the coarse levels that run as one cluster launch
-  const int prec = H->opt.precision == 1 ? kFP32 : kFP64;
-  for (int o = 1; o <= 2; ++o) {
-    H->cl_plan[o] = ClPlan();
-    if (!cluster_runs(H)) continue;
-    H->cl_plan[o] = cluster_plan(H->L, H->deepest[o], o, prec, H->cl_bound);
-    if (H->cl_plan[o].first)
-      CKS(launch_ok(H, launch_cluster_build(H->L, H->cl_plan[o], o, prec, H->cl_blobs[o], s), "coarse-level records"));
-  }
+  // the coarse levels that run as one cluster launch (a batch's patch: once a
+  // cycle of its own asks for them)
+  H->cl_stale = true;
+  if (!H->patch) CKS(build_cluster(H));
   // the coarsest solve's map of each order, for the bottom cycle (one launch)
   const LevelDev* mapped[3] = {nullptr, nullptr, nullptr};
   for (int o = 1; o <= 2; ++o) {
@@ -789,6 +813,7 @@ void destroy(mg_hierarchy* H) {
   if (H->cap_stream) cudaStreamDestroy(H->cap_stream);
   if (H->staging) cudaFree(H->staging);
   if (H->arena) cudaFree(H->arena);
+  if (H->cl_own) cudaFree(H->cl_own);
   if (H->hscal) cudaFreeHost(H->hscal);
   if (H->own_stream && H->stream) cudaStreamDestroy(H->stream);
   delete H;
@@ -897,6 +922,13 @@ int mg_checked_build(void) {
 
 mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, int nz, double h,
                               const mg_options* opt, void* cuda_stream, mg_hierarchy** out) {
+  return create_hierarchy(mask, where, nx, ny, nz, h, opt, cuda_stream, false, out);
+}
+
+}  // extern "C"
+
+mg_status gbmg::create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, int nz, double h,
+                                 const mg_options* opt, void* cuda_stream, bool patch, mg_hierarchy** out) {
   if (out) *out = nullptr;
   if (!out || !mask) return fail(nullptr, MG_ERR_INVALID_ARG, "null mask or output pointer");
   if (where != MG_MEM_HOST && where != MG_MEM_DEVICE) return fail(nullptr, MG_ERR_INVALID_ARG, "bad mg_mem");
@@ -916,6 +948,7 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
 
   mg_hierarchy* H = new mg_hierarchy();
   H->opt = o;
+  H->patch = patch;
   H->h = h;
   if (cudaGetDevice(&H->device) != cudaSuccess) {
     delete H;
@@ -997,9 +1030,12 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
         if (cluster_level(H->L[l].g)) info += sizeof(uint32_t) * (H->L[l].g.nz + 1);
       }
   const size_t o_info = A.reserve(info);
-  H->cl_bound = H->cluster_ok ? cluster_blob_bound(H->L, H->nlev, mixed ? kFP32 : kFP64) : 0;
+  // the cluster's records, where its launches can run
+  if (!patch && cluster_runs(H)) H->cl_bound = cluster_blob_bound(H->L, H->nlev, mixed ? kFP32 : kFP64);
   size_t o_blobs[3] = {0, 0, 0};
-  for (int ord = 1; ord <= 2; ++ord) o_blobs[ord] = A.reserve(H->cl_bound);
+  auto has_blobs = [&](int ord) { return H->cl_bound > 0 && (o.order == 0 || o.order == ord); };
+  for (int ord = 1; ord <= 2; ++ord)
+    if (has_blobs(ord)) o_blobs[ord] = A.reserve(H->cl_bound);
   // batched build launches: one scratch word per list block of every list
   std::vector<ListJob> ljobs;
   unsigned lblocks = 0;
@@ -1073,7 +1109,8 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
     return st;
   }
   char* base = H->arena;
-  for (int ord = 1; ord <= 2; ++ord) H->cl_blobs[ord] = base + o_blobs[ord];
+  for (int ord = 1; ord <= 2; ++ord)
+    if (has_blobs(ord)) H->cl_blobs[ord] = base + o_blobs[ord];
   H->build_info = base + o_info;
   H->build_info_bytes = info;
   H->hbuild_info = (const char*)(H->hscal + 8);
@@ -1192,6 +1229,8 @@ mg_status mg_create_hierarchy(const int8_t* mask, mg_mem where, int nx, int ny, 
   *out = H;
   return MG_OK;
 }
+
+extern "C" {
 
 mg_status mg_destroy_hierarchy(mg_hierarchy* H) {
   destroy(H);
