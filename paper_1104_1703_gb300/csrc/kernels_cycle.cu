@@ -1233,8 +1233,10 @@ cudaError_t prolong_t(const LevelDev& Lc, const LevelDev& Lf, int order, bool bl
   count_launch();
   if constexpr (sizeof(T) == 8) {
     // two unknowns per thread where that leaves every SM its threads (at 240
-    // thousand unknowns W-cycles are 0.5% slower with it)
-    if (Lf.level == 0 && n >= 8u * (uint32_t)device_sms() * kListBlock) {
+    // thousand unknowns W-cycles are 0.5% slower with it) and rows are long
+    // enough for neighbours in most pairs (2.5 million unknowns, rows of 8 cells
+    // 45.9 us, one per thread 57.4; of 6 cells 65.2 and 57.8, of 2 115 and 108)
+    if (Lf.level == 0 && Lf.g.hx >= 4 && n >= 8u * (uint32_t)device_sms() * kListBlock) {
       launch_pdl(prolong_list_pairs_kernel, dim3(exact_grid((n + 3) / 2, 1)), dim3(kListBlock), 0, s, a);
       return cudaGetLastError();
     }
