@@ -526,8 +526,7 @@ bool make_conv_input_map(CUtensorMap* map, const __nv_bfloat16* x, int W, int H,
   const cuuint32_t box[5] = {(cuuint32_t)span, (cuuint32_t)bx, (cuuint32_t)by, (cuuint32_t)bz, (cuuint32_t)blocks};
   const CUtensorMapSwizzle sw = span == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
                                 : span == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
-                                : span == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
-                                             : CU_TENSOR_MAP_SWIZZLE_NONE;
+                                             : CU_TENSOR_MAP_SWIZZLE_32B;
   const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)x, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==

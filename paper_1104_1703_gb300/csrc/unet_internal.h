@@ -65,8 +65,8 @@ size_t conv_smem_bytes(const ConvArgs& a);
 __host__ __device__ uint32_t conv_tmem_cols(int group, int cout);
 cudaError_t init_conv_kernel(size_t smem_bytes);
 // `map` describes the input tensor: dims (span, W, H, D, cin / span), box
-// (span, bx, by, bz, blocks), BF16, swizzled over rows of `span` channels
-// (span 8: no swizzle).
+// (span, bx, by, bz, blocks), BF16, swizzled over rows of `span` channels (64,
+// 32 or 16).
 bool make_conv_input_map(CUtensorMap* map, const __nv_bfloat16* x, int W, int H, int D, int cin, int span, int bx,
                          int by, int bz, int blocks);
 bool make_conv_map(CUtensorMap* map, const __nv_bfloat16* x, const ConvArgs& a);
