@@ -423,8 +423,11 @@ def roofline(st, n_active, precision, peaks, fp64_rate=None, pass_on=False, seg_
         # 25 B per update over the red+black sweep: read the other colour 8,
         # b/D 8, code 1, write 8.  The method's 7 FP64 operations per update
         # (6 adds, 1 multiply) issue as 1 fused multiply-add when the
-        # neighbour sum is formed in integer arithmetic (fp64_sum), else 6
+        # neighbour sum is formed in integer arithmetic (fp64_sum), else 6;
+        # the integer sum's rounding, an integer-to-double conversion, takes
+        # the FP64 pipe as well
         ops = 1.0 if exact_on else 6.0
+        pipe = 2.0 if exact_on else 6.0
         if fp64_rate:
             peak, psrc = fp64_rate / 1e12, "measured DFMA rate on this GPU (mg_probe_fp64_rate)"
         else:
@@ -439,6 +442,8 @@ def roofline(st, n_active, precision, peaks, fp64_rate=None, pass_on=False, seg_
                 "launches": st["gs_n"], "avg_launch_us": gs_s * 1e6, "peak_source": src,
                 "fp64_pipe_view": {"achieved": ops * half / gs_s / 1e12, "peak": peak, "unit": "T FP64 instr/s",
                                    "frac": ops * half / gs_s / 1e12 / peak, "issued_fp64_ops_per_update": ops,
+                                   "pipe_instructions_per_update": pipe,
+                                   "pipe_frac": pipe * half / gs_s / 1e12 / peak,
                                    "method_fp64_ops_per_update": 7, "peak_source": psrc}}
     # FP32: read the other colour 4 + b 4 + code 1, write 4 = 13 B per update
     if pass_on:

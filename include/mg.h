@@ -109,7 +109,8 @@ typedef enum { MG_MEM_HOST = 0, MG_MEM_DEVICE = 1 } mg_mem;
  *                  of its six neighbour values in 64-bit integer arithmetic
  *                  (exponent-aligned fixed point, rounded once to the
  *                  nearest double; subnormal values count as zero), so that
- *                  a sweep's update issues one FP64 instruction instead of
+ *                  a sweep's update issues two instructions to the FP64 pipe
+ *                  (the sum's rounding and a multiply-add) instead of
  *                  six; 0 = five FP64 additions.  Both are accurate to about
  *                  one rounding of the sum; the results differ in the last
  *                  bits.

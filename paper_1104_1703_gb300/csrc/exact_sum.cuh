@@ -1,7 +1,8 @@
-// Sum of a few doubles without the FP64 pipe: the FP64 level-0 sweep's
+// Sum of a few doubles without FP64 additions: the FP64 level-0 sweep's
 // neighbour sum (Section 2's 7-point stencil: the six neighbour values of a
-// cell) formed with integer instructions, so that the sweep issues one FP64
-// instruction per update (the final multiply-add) instead of six.
+// cell) formed with integer instructions, so that the sweep issues two
+// instructions to the FP64 pipe per update (the conversion that rounds the sum,
+// and the final multiply-add) instead of six.
 //
 // Method: fixed-point accumulation in one 64-bit window anchored at the
 // largest exponent of the terms (a narrow form of Kulisch's long

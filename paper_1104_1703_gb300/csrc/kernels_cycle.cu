@@ -1839,7 +1839,8 @@ cudaError_t launch_refine_residual(const LevelDev& L0, double* partials, int max
   if (blocks > max_partials) return cudaErrorInvalidValue;
   count_launch();
   if (L0.exact_sum) launch_pdl(refine_residual_kernel<true>, dim3(blocks), dim3(kListBlock), 0, s, a);
-  else launch_pdl(refine_residual_kernel<false>, dim3(blocks), dim3(kListBlock), 0, s, a);  launch_finalize(partials, blocks, out, loop, s);
+  else launch_pdl(refine_residual_kernel<false>, dim3(blocks), dim3(kListBlock), 0, s, a);
+  launch_finalize(partials, blocks, out, loop, s);
   return cudaGetLastError();
 }
 

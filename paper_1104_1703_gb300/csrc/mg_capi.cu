@@ -739,7 +739,7 @@ mg_status build_levels(mg_hierarchy* H, bool fine_built = false, const int8_t* m
     CKS(launch_ok(H, launch_coarse_coeffs(H->L[l + 1], H->counts + 2 * (l + 1), s), "coarse coefficients"));
   }
   // compact lists of the unknowns, per order and colour (level 0: one set),
-  // all in three launches
+  // all in four launches
   CKS(launch_ok(H, launch_build_lists(H->list_jobs, H->n_list_jobs, H->list_blocks, H->list_scratch, s),
                 "active lists"));
   if (H->pass_on)

@@ -251,9 +251,7 @@ cudaError_t launch_restrict(const LevelDev& Lf, const LevelDev& Lc, int order, b
 // which overwrites the red ones without reading them).
 cudaError_t launch_prolong(const LevelDev& Lc, const LevelDev& Lf, int order, int prec, bool black_only,
                            cudaStream_t s);
-// Sum of squares of the scaled residual of level 0 into partials[0..nblocks),
-// then a fixed-order reduction into out[0].  red_only as black_zero above.
-// with_phi = false evaluates the residual of Phi = 0 (i.e. of the rhs alone).
+
 // State of a solve's cycles run as one graph (a conditional while node): the
 // host writes it, the finalize kernel of every cycle adds the cycle's residual
 // norm and decides, by the host's rule and in its arithmetic, whether another
@@ -278,6 +276,9 @@ struct LoopEnd {
   cudaGraphConditionalHandle handle = 0;
 };
 
+// Sum of squares of the scaled residual of level 0 into partials[0..nblocks),
+// then a fixed-order reduction into out[0].  red_only as black_zero above.
+// with_phi = false evaluates the residual of Phi = 0 (i.e. of the rhs alone).
 cudaError_t launch_residual_norm2(const LevelDev& L0, bool red_only, bool with_phi, double* partials,
                                   int max_partials, double* out, cudaStream_t s, LoopEnd loop = LoopEnd());
 // One multigrid iteration with n_cycles coarse iterations per level (1: V,
