@@ -96,3 +96,23 @@ def test_fold(shape, p_active):
                 H.set_dirichlet_from_coarse(phi_c, (-2, 0, -2))
     # the same six terms added in another order at most: 6 roundings of values below 12 max|phi_c|
     assert np.abs(got - want).max() <= 6 * 2.0 ** -52 * 12 * float(phi_c.abs().max())
+
+
+@pytest.mark.parametrize("shape", [(200, 300, 3), (20, 22, 140)])
+@pytest.mark.parametrize("value", [float("inf"), float("nan")])
+def test_fold_non_finite(shape, value):
+    """A non-finite coarse value reaches the cells whose faces it serves, and no other."""
+    nz, ny, nx = shape
+    mask, rho, _, faces = _fields(shape, 15, 0.9)
+    phi_c = torch.ones(tuple((n + 1) // 2 + 2 for n in shape), dtype=torch.float64, device="cuda")
+    phi_c[nz // 4, ny // 4, 1] = value
+    with B.Hierarchy(mask, 0.125) as H:
+        H.set_rhs(rho)
+        H.set_dirichlet_from_coarse(phi_c, (-2, -2, -2))
+        got = H.level_get(0, B.MG_FIELD_RHS)
+        H.faces_from_coarse(phi_c, (-2, -2, -2), *faces)
+        H.set_dirichlet(*faces)
+        want = H.level_get(0, B.MG_FIELD_RHS)
+    bad = ~np.isfinite(got)
+    assert 0 < bad.sum() < 2000 and np.array_equal(bad, ~np.isfinite(want))
+    assert np.abs(got[~bad] - want[~bad]).max() <= 6 * 2.0 ** -52 * (12 + 0.02 * float(rho.abs().max()))
